@@ -204,8 +204,12 @@ omprt_status omprt_alloc_shared(omprt_ctx *ctx, size_t bytes_per_team);
  * stencils (no reduction, n and nx multiples of 4) stage an input window that
  * reaches one element / one row beyond the pass, when the chunk is at most
  * 512 bytes and the two halos at most a quarter of the pass.  A claim of 32
- * chunks runs in equal passes.  Other launches, and teams whose block does
- * not start on a 16-byte boundary, run the plain form.  The 2-D stencil under
+ * chunks runs in equal passes.  Streaming bodies whose blocks do not all
+ * start on a 16-byte boundary, or whose passes do not fit, take the row form
+ * where their pieces are long enough (128 bytes under static(c) and
+ * dynamic(c), 256 under static): each lane's next 64 or 128 bytes of its piece
+ * at a time, in buffers sized from the device's shared memory, whatever
+ * `bytes`.  Other launches run the plain form.  The 2-D stencil under
  * static(c) with c in [4, 8) or [32, 128] (fp32, no reduction, nx a multiple of
  * 4, n < 2^32, 16-byte-aligned pointers) instead walks each team's block in
  * passes of two rows through a six-row ring in shared memory (six rows of nx

@@ -341,6 +341,77 @@ static StagePlan stage_plan(const omprt_ctx* c, const StageShape& sh, uint64_t c
   return {(uint32_t)P, (uint32_t)wb};
 }
 
+// The row form (region_rows.cuh) of a launch whose threads run contiguous
+// pieces.  It takes the launches below, measured on GB300 with axpy and dot at
+// n = 2^18 .. 2^26 (plain -> rows; G x T teams x threads):
+//   - pieces of 128 bytes on under static(c) and dynamic(c) (static(32)
+//     608 x 256: 260 -> 150 us, static(64) 191 -> 135; static(16) 232 -> 236),
+//     of 256 under static, whose short pieces still share lines (53 elements
+//     26.1 -> 28.4 us, 110 elements 45.9 -> 43.1);
+//   - blocks of 16 chunks on: with fewer, most lanes of the only claim are
+//     idle and each walks its chunk slab by slab (7 chunks of 256:
+//     11.2 -> 12.6 us; 27 chunks: 19.4 -> 13.4);
+//   - not static with a compensated sum: there the adds, not the loads, hold a
+//     launch (dot 500 x 512: 101 -> 111 us), unless the pieces are long;
+//   - a single stage a warp (teams of 1024) only where the plain form is
+//     worst: pieces of 512 bytes on (dynamic(256) 333 x 1024: 261 -> 164 us;
+//     static(64) 156 -> 175).
+// Shape: rows of 128 bytes where two stages a warp fit, else of 64; 64 also
+// for compensated sums, which want more warps (dot dynamic(256): 112 -> 103
+// us).  CTAs an SM: the count whose last wave is fullest, among those that
+// keep enough in flight (14 stages of 128-byte rows an SM; 608 x 256: one CTA
+// with two stages a warp 139 us, two with one 153).  Sized from the device's
+// shared memory, whatever the staging bytes; those at zero turn it off.
+struct RowPlan {
+  uint32_t row_bytes, stages;  // row_bytes 0: not this form
+  size_t smem;                 // dynamic shared memory of the buffers
+};
+static RowPlan row_plan(const omprt_ctx* c, const omprt_loop_desc* d, const StageShape& sh,
+                        uint64_t n, int ksched, uint64_t chunk, uint32_t teams, uint32_t threads,
+                        size_t smem_base, bool comp_sum) {
+  RowPlan best = {0u, 0u, 0};
+  if (!sh.arrays || sh.halo || c->stage_bytes == 0 || n == 0) return best;
+  uintptr_t mis = (uintptr_t)d->x;
+  if (sh.arrays == 2) mis |= (uintptr_t)d->y;
+  if (mis & 15) return best;
+  const bool whole = ksched == kStatic;  // one piece a thread
+  const uint64_t block = (n - 1) / teams + 1;
+  const uint64_t piece = (whole ? block / threads : chunk) * sh.elem;
+  if (piece < (whole ? (comp_sum ? 2048u : 256u) : 128u)) return best;
+  uint32_t warps = threads / 32;  // that can be busy at once
+  if (!whole) {
+    const uint64_t chunks = (block - 1) / chunk + 1;
+    if (chunks < 16) return best;
+    if ((chunks + 31) / 32 < warps) warps = (uint32_t)((chunks + 31) / 32);
+  }
+  constexpr uint64_t kStatic_ = 2048;      // the kernels' static shared memory, rounded up
+  constexpr uint64_t kReserved = 1024;     // what the hardware keeps of it for each CTA
+  const uint32_t most = threads >= 1024 ? 1 : 1024 / threads;  // CTAs an SM, by registers
+  double top = 0;
+  for (uint32_t row = comp_sum ? 64 : 128; row >= 64 && !best.row_bytes; row /= 2) {
+    const uint64_t set = (uint64_t)warps * rt::row_stage_bytes(sh.arrays, row);
+    for (uint32_t k = most; k >= 1; --k) {
+      uint64_t room = (uint64_t)c->smem_per_sm / k;
+      if (room > (uint64_t)c->max_smem_optin + kReserved) room = (uint64_t)c->max_smem_optin + kReserved;
+      const uint64_t fixed = kReserved + kStatic_ + smem_base;
+      uint64_t ns = room > fixed ? (room - fixed) / set : 0;
+      if (ns > rt::kRowStagesMax) ns = rt::kRowStagesMax;
+      if (ns == 0 || (ns == 1 && row == 128)) continue;
+      if (ns == 1 && threads >= 1024 && piece < 512) continue;
+      const double wave = (double)c->sm_count * k;
+      const double full = teams / wave / std::ceil(teams / wave);
+      const double flight = (double)(k * warps * ns) * row / (14 * 128), busy = k * warps / 16.0;
+      double score = full * std::fmin(flight, 1.0) * (ns > 1 ? 1.0 : 0.92);
+      if (comp_sum) score *= std::fmin(busy, 1.0);
+      if (score > top * 1.001) {
+        top = score;
+        best = {row, (uint32_t)ns, (size_t)(ns * set)};
+      }
+    }
+  }
+  return best;
+}
+
 static omprt_status launch_region_impl(omprt_ctx* c, const omprt_loop_desc* d, int64_t dist_chunk,
                                        int32_t sched, int64_t chunk, int32_t teams,
                                        int32_t threads, const omprt_reduce_desc* red,
@@ -438,8 +509,13 @@ static omprt_status launch_region_impl(omprt_ctx* c, const omprt_loop_desc* d, i
   if (ksched == kDynamic || ksched == kChunked || ksched == kNonmono) stage_c = (uint64_t)chunk;
   if (ksched == kStatic && n % ((uint64_t)teams * (uint64_t)threads) == 0)
     stage_c = n / ((uint64_t)teams * (uint64_t)threads);
-  if (stage_c) {
-    const StagePlan sp = stage_plan(c, stage_shape(d, n), stage_c, (uint32_t)threads, smem,
+  const StageShape sh = stage_shape(d, n);
+  // the staged form runs in blocks that start on a 16-byte boundary; where
+  // not all do, streaming bodies take the row form instead (axpy static(64)
+  // at n = 2^26, 900 x 128: 227 -> 139 us)
+  const bool aligned = n % (uint64_t)teams == 0 && n / (uint64_t)teams * sh.elem % 16 == 0;
+  if (stage_c && (aligned || sh.halo)) {
+    const StagePlan sp = stage_plan(c, sh, stage_c, (uint32_t)threads, smem,
                                     acc != kAccNone);
     if (sp.chunks) {
       a.stage_chunks = sp.chunks;
@@ -447,6 +523,17 @@ static omprt_status launch_region_impl(omprt_ctx* c, const omprt_loop_desc* d, i
       a.stage_off = (uint32_t)smem;
       if (ksched == kStatic) a.chunk = stage_c;
       smem += (size_t)(threads / 32) * sp.warp_bytes;
+    }
+  }
+  if (!a.stage_chunks && (ksched == kStatic || ksched == kChunked || ksched == kDynamic ||
+                          ksched == kNonmono)) {
+    const RowPlan rp = row_plan(c, d, sh, n, ksched, (uint64_t)chunk,
+                                (uint32_t)teams, (uint32_t)threads, smem, acc == kAccCompF32);
+    if (rp.row_bytes) {
+      a.row_bytes = rp.row_bytes;
+      a.row_stages = rp.stages;
+      a.stage_off = (uint32_t)smem;
+      smem += rp.smem;
     }
   }
   cudaStream_t st = (cudaStream_t)stream;

@@ -8,6 +8,15 @@ namespace rt {
 template <class Body, class Acc, int SCHED>
 inline cudaError_t launch_one(unsigned grid, unsigned block, size_t smem, cudaStream_t st,
                               const RegionArgs& a) {
+  if constexpr (rows_for<Body, SCHED>()) {
+    if (a.row_bytes) {
+      auto k = rows_kernel<Body, SCHED, Acc>;
+      static const size_t static_bytes = static_smem_of(k);
+      const cudaError_t e = smem_optin(k, smem, static_bytes);
+      if (e != cudaSuccess) return e;
+      return launch_kernel(k, grid, block, smem, st, a);
+    }
+  }
   auto k = region_kernel<Body, SCHED, Acc>;
   static const size_t static_bytes = static_smem_of(k);
   const cudaError_t e = smem_optin(k, smem, static_bytes);

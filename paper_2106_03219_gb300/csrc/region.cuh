@@ -53,6 +53,8 @@ struct RegionArgs {
   uint32_t stage_chunks;  // staged schedules: chunks per pass (0: the plain form)
   uint32_t stage_off;     // byte offset of the staging buffers in dynamic shared memory
   uint32_t stage_warp_bytes;  // staging buffer bytes per warp
+  uint32_t row_bytes;   // row form: bytes a row, 64 or 128 (0: not this form)
+  uint32_t row_stages;  // row form: stages a warp
   unsigned char* partials;        // 16 bytes per team
   uint32_t* ticket;               // cross-team ticket (wraps to 0 by itself)
   unsigned long long* dyn_next;   // per-team dynamic dispatch counters (left 0)
@@ -137,13 +139,13 @@ struct BodyAxpyF32 {
   __device__ const void* stage_src(int k) const { return k ? (const void*)y : (const void*)x; }
   __device__ void* stage_dst() const { return y; }
   template <class Acc>
-  __device__ __forceinline__ void stage_unit(uint4 (&u)[2], Acc& acc) const {
+  __device__ __forceinline__ void stage_unit(uint4 (&u)[2], Acc& acc, uint32_t mask = ~0u) const {
     u[1].x = as_u(__fmaf_rn(a, as_f(u[0].x), as_f(u[1].x)));
     u[1].y = as_u(__fmaf_rn(a, as_f(u[0].y), as_f(u[1].y)));
     u[1].z = as_u(__fmaf_rn(a, as_f(u[0].z), as_f(u[1].z)));
     u[1].w = as_u(__fmaf_rn(a, as_f(u[0].w), as_f(u[1].w)));
-    acc_add2(acc, as_f(u[1].x), as_f(u[1].y));
-    acc_add2(acc, as_f(u[1].z), as_f(u[1].w));
+    acc_add2(acc, as_f(u[1].x), as_f(u[1].y), mask);
+    acc_add2(acc, as_f(u[1].z), as_f(u[1].w), mask >> 2);
   }
 };
 
@@ -187,15 +189,15 @@ struct BodyAxpyI32 {
   __device__ const void* stage_src(int k) const { return k ? (const void*)y : (const void*)x; }
   __device__ void* stage_dst() const { return y; }
   template <class Acc>
-  __device__ __forceinline__ void stage_unit(uint4 (&u)[2], Acc& acc) const {
+  __device__ __forceinline__ void stage_unit(uint4 (&u)[2], Acc& acc, uint32_t mask = ~0u) const {
     u[1].x = a * u[0].x + u[1].x;
     u[1].y = a * u[0].y + u[1].y;
     u[1].z = a * u[0].z + u[1].z;
     u[1].w = a * u[0].w + u[1].w;
-    acc.add((int32_t)u[1].x);
-    acc.add((int32_t)u[1].y);
-    acc.add((int32_t)u[1].z);
-    acc.add((int32_t)u[1].w);
+    if (mask & 1) acc.add((int32_t)u[1].x);
+    if (mask & 2) acc.add((int32_t)u[1].y);
+    if (mask & 4) acc.add((int32_t)u[1].z);
+    if (mask & 8) acc.add((int32_t)u[1].w);
   }
 };
 
@@ -235,9 +237,11 @@ struct BodyDotF32 {
   __device__ const void* stage_src(int k) const { return k ? (const void*)y : (const void*)x; }
   __device__ void* stage_dst() const { return nullptr; }
   template <class Acc>
-  __device__ __forceinline__ void stage_unit(uint4 (&u)[2], Acc& acc) const {
-    acc_add2(acc, __fmul_rn(as_f(u[0].x), as_f(u[1].x)), __fmul_rn(as_f(u[0].y), as_f(u[1].y)));
-    acc_add2(acc, __fmul_rn(as_f(u[0].z), as_f(u[1].z)), __fmul_rn(as_f(u[0].w), as_f(u[1].w)));
+  __device__ __forceinline__ void stage_unit(uint4 (&u)[2], Acc& acc, uint32_t mask = ~0u) const {
+    acc_add2(acc, __fmul_rn(as_f(u[0].x), as_f(u[1].x)), __fmul_rn(as_f(u[0].y), as_f(u[1].y)),
+             mask);
+    acc_add2(acc, __fmul_rn(as_f(u[0].z), as_f(u[1].z)), __fmul_rn(as_f(u[0].w), as_f(u[1].w)),
+             mask >> 2);
   }
 };
 
@@ -267,9 +271,9 @@ struct BodyLoadF32 {
   __device__ const void* stage_src(int) const { return x; }
   __device__ void* stage_dst() const { return nullptr; }
   template <class Acc>
-  __device__ __forceinline__ void stage_unit(uint4 (&u)[1], Acc& acc) const {
-    acc_add2(acc, as_f(u[0].x), as_f(u[0].y));
-    acc_add2(acc, as_f(u[0].z), as_f(u[0].w));
+  __device__ __forceinline__ void stage_unit(uint4 (&u)[1], Acc& acc, uint32_t mask = ~0u) const {
+    acc_add2(acc, as_f(u[0].x), as_f(u[0].y), mask);
+    acc_add2(acc, as_f(u[0].z), as_f(u[0].w), mask >> 2);
   }
 };
 
@@ -305,10 +309,11 @@ struct BodyLoadBF16 {
   __device__ const void* stage_src(int) const { return x; }
   __device__ void* stage_dst() const { return nullptr; }
   template <class Acc>
-  __device__ __forceinline__ void stage_unit(uint4 (&u)[1], Acc& acc) const {
+  __device__ __forceinline__ void stage_unit(uint4 (&u)[1], Acc& acc, uint32_t mask = ~0u) const {
     const uint32_t w[4] = {u[0].x, u[0].y, u[0].z, u[0].w};
 #pragma unroll
-    for (int k = 0; k < 4; ++k) acc_add2(acc, as_f(w[k] << 16), as_f(w[k] & 0xffff0000u));
+    for (int k = 0; k < 4; ++k)
+      acc_add2(acc, as_f(w[k] << 16), as_f(w[k] & 0xffff0000u), mask >> (2 * k));
   }
 };
 
@@ -337,11 +342,11 @@ struct BodyLoadI32 {
   __device__ const void* stage_src(int) const { return x; }
   __device__ void* stage_dst() const { return nullptr; }
   template <class Acc>
-  __device__ __forceinline__ void stage_unit(uint4 (&u)[1], Acc& acc) const {
-    acc.add((int32_t)u[0].x);
-    acc.add((int32_t)u[0].y);
-    acc.add((int32_t)u[0].z);
-    acc.add((int32_t)u[0].w);
+  __device__ __forceinline__ void stage_unit(uint4 (&u)[1], Acc& acc, uint32_t mask = ~0u) const {
+    if (mask & 1) acc.add((int32_t)u[0].x);
+    if (mask & 2) acc.add((int32_t)u[0].y);
+    if (mask & 4) acc.add((int32_t)u[0].z);
+    if (mask & 8) acc.add((int32_t)u[0].w);
   }
 };
 
@@ -370,9 +375,9 @@ struct BodyLoadI64 {
   __device__ const void* stage_src(int) const { return x; }
   __device__ void* stage_dst() const { return nullptr; }
   template <class Acc>
-  __device__ __forceinline__ void stage_unit(uint4 (&u)[1], Acc& acc) const {
-    acc.add((int64_t)(((uint64_t)u[0].y << 32) | u[0].x));
-    acc.add((int64_t)(((uint64_t)u[0].w << 32) | u[0].z));
+  __device__ __forceinline__ void stage_unit(uint4 (&u)[1], Acc& acc, uint32_t mask = ~0u) const {
+    if (mask & 1) acc.add((int64_t)(((uint64_t)u[0].y << 32) | u[0].x));
+    if (mask & 2) acc.add((int64_t)(((uint64_t)u[0].w << 32) | u[0].z));
   }
 };
 
@@ -1347,3 +1352,5 @@ __global__ void __launch_bounds__(OMPRT_MAX_THREADS) region_kernel(const RegionA
 }
 
 }  // namespace rt
+
+#include "region_rows.cuh"

@@ -530,15 +530,17 @@ struct AccCompF32 {
 };
 
 // Feed a, b (in this order) to an accumulator: packed where it has a pair
-// form, else two adds.
+// form, else two adds.  mask bits 0 and 1: whether a and b take part.
 template <class Acc>
-__device__ __forceinline__ void acc_add2(Acc& acc, float a, float b) {
+__device__ __forceinline__ void acc_add2(Acc& acc, float a, float b, uint32_t mask = 3u) {
   if constexpr (std::is_same<Acc, AccCompF32>::value) {
-    acc.add2(a, b);
-  } else {
-    acc.add(a);
-    acc.add(b);
+    if ((mask & 3u) == 3u) {
+      acc.add2(a, b);
+      return;
+    }
   }
+  if (mask & 1u) acc.add(a);
+  if (mask & 2u) acc.add(b);
 }
 
 struct AccNaiveF32 {
