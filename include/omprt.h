@@ -323,9 +323,11 @@ omprt_status omprt_launch_region_dist(omprt_ctx *ctx, const omprt_loop_desc *des
  * id, its loop bounds, its arguments: the scale and a pointer to the
  * globalised reduction variable) and releases the waiting workers; every
  * thread dispatches on the id and runs the region's parallel for (the
- * default schedule: static with a chunk of one 32-byte vector) with a
- * compensated reduction into the variable; a join barrier returns control to
- * the main thread.  Globalised variables live on the team stack of capacity
+ * default schedule: static with a chunk of one 32-byte vector, or of one
+ * 16-byte unit where the team streams its segments through tiles in the
+ * shared memory its stack leaves: teams of up to 480 threads, x and y 16-byte
+ * aligned) with a compensated reduction into the variable; a join barrier
+ * returns control to the main thread.  Globalised variables live on the team stack of capacity
  * S (omprt_alloc_shared), overflowing to the team's 4 KiB pool slice (teams
  * below OMPRT_MAX_RED_TEAMS); a request that does not fit sets
  * OMPRT_DEV_STACK_NOMEM and the team stops (its remaining results are not

@@ -384,20 +384,30 @@ __device__ __forceinline__ void bulk_wait_all() {
 __device__ __forceinline__ void fence_proxy_async() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
+// Whether phase `phase` of the mbarrier has completed, suspended for up to
+// 20 us instead of spinning.
+__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t phase) {
+  uint32_t done;
+  asm volatile(
+      "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3; selp.u32 %0, "
+      "1, 0, p; }"
+      : "=r"(done)
+      : "r"(bar), "r"(phase), "r"(20000u)
+      : "memory");
+  return done != 0;
+}
 // Wait for phase `phase` of the mbarrier to complete, for at most max_ns of
 // the global timer; on expiry set the timeout bit (if status) and return false.
-__device__ inline bool mbar_wait(uint32_t bar, uint32_t phase, uint64_t max_ns, uint32_t* status) {
+// The timer is read only once a try has run out.  stop (if given): a
+// team-shared flag that also ends the wait (false, no bit).
+__device__ inline bool mbar_wait(uint32_t bar, uint32_t phase, uint64_t max_ns, uint32_t* status,
+                                 const volatile int* stop = nullptr) {
+  if (mbar_try(bar, phase)) return true;
   uint64_t t0;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
   for (;;) {
-    uint32_t done;
-    asm volatile(
-        "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3; selp.u32 %0, "
-        "1, 0, p; }"
-        : "=r"(done)
-        : "r"(bar), "r"(phase), "r"(20000u)  // suspend up to 20 us per try instead of spinning
-        : "memory");
-    if (done) return true;
+    if (mbar_try(bar, phase)) return true;
+    if (stop && *stop) return false;
     uint64_t t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     if (t - t0 > max_ns) {

@@ -131,3 +131,43 @@ def test_generic_out_of_stack_flagged(rt):
     rt.launch_generic(dev(seg[:2]), R.loop_desc(R.BODY_DOT, n=n, x=dev(x), y=dev(y), alpha=0.5),
                       res2, 1, 32, program=R.GENERIC_DOT_AXPY)
     assert rt.sync_status() == 0
+
+
+# The tiled form: segments of no, one, as many and more tiles than the ring
+# holds (a tile is at most 8192 elements, three fit), starting at every place of a
+# 16-byte unit, up to an array end inside one; long runs of empty segments;
+# teams beyond the segments; and arrays no form but the plain one takes.
+@pytest.mark.parametrize("G,T", [(1, 32), (2, 256), (7, 480), (300, 64), (2, 512)])
+@pytest.mark.parametrize("off", [0, 4, 1])
+def test_generic_tiles(rt, G, T, off):
+    import torch
+    lens = [0, 1, 2, 3, 4, 5, 8191, 8192, 8193, 0, 0, 0, 24575, 24576, 24577, 1, 60001, 0, 33,
+            14337, 100003]
+    seg = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    n, nseg = int(seg[-1]), len(lens)
+    xb, yb = inputs.f32_uniform01(n + 8, 0), inputs.f32_uniform01(n + 8, 1)
+    x, y = xb[off:off + n], yb[off:off + n]
+    xd, yd = dev(xb), dev(yb)
+    xv, yv = xd[off:off + n], yd[off:off + n]
+    res = torch.full((3 * nseg,), -1.0, dtype=torch.float64, device="cuda")
+    rt.launch_generic(dev(seg), R.loop_desc(R.BODY_DOT, n=n, x=xv, y=yv), res[:nseg], G, T)
+    got = host(res)
+    for s in range(nseg):
+        exact = O.exact_dot_f32(x[seg[s]:seg[s + 1]], y[seg[s]:seg[s + 1]])
+        assert abs(got[s] - exact) <= 1e-6 * max(abs(exact), 1e-300), s
+    rt.launch_generic(dev(seg), R.loop_desc(R.BODY_DOT, n=n, x=xv, y=yv, alpha=1e-4), res, G, T,
+                      program=R.GENERIC_DOT_AXPY)
+    got, ynew = host(res), host(yd)
+    assert np.array_equal(bits32(ynew[:off]), bits32(yb[:off]))
+    assert np.array_equal(bits32(ynew[off + n:]), bits32(yb[off + n:]))
+    for s in range(nseg):
+        xs, ys = x[seg[s]:seg[s + 1]], y[seg[s]:seg[s + 1]]
+        exact = O.exact_dot_f32(xs, ys)
+        assert abs(got[3 * s] - exact) <= 1e-6 * max(abs(exact), 1e-300), s
+        a = np.float32(np.float32(got[3 * s]) * np.float32(1e-4))
+        assert got[3 * s + 1] == float(a), s
+        want = O.axpy_f32(float(a), xs, ys)
+        assert np.array_equal(bits32(ynew[off + seg[s]:off + seg[s + 1]]), bits32(want)), s
+        exact = O.exact_sum_f32(want)
+        assert abs(got[3 * s + 2] - exact) <= 1e-6 * max(abs(exact), 1e-300), s
+    assert rt.sync_status() == 0
