@@ -535,7 +535,7 @@ omprt_status omprt_mlp_forward(omprt_ctx *ctx, const float *params_dev, const fl
 /* (Learned schedule: this library's own, not a routine of the paper's
  * runtime.)  Mean-squared-error loss over the batch and the 12 outputs and its gradient:
  * grad_dev[6028] = d loss / d params (overwritten), loss_dev[1] (may be NULL).
- * batch in [1, 16384]; the per-sample activations go to context scratch, so
+ * batch in [1, 16384]; the partial gradients go to context scratch, so
  * calls on one context must not overlap on the device. */
 omprt_status omprt_mlp_loss_grad(omprt_ctx *ctx, const float *params_dev, const float *x_dev,
                                  const float *target_dev, int32_t batch, float *grad_dev,

@@ -189,7 +189,7 @@ omprt_status omprt_init(int device, omprt_ctx** out) {
             cudaMalloc(&c->slots_dev, kSlotBytes * OMPRT_SLOTS) == cudaSuccess &&
             cudaMalloc(&c->pool_dev, (size_t)OMPRT_MAX_RED_TEAMS * OMPRT_POOL_BYTES_PER_TEAM) ==
                 cudaSuccess &&
-            cudaMalloc(&c->mlp_rows_dev, sizeof(float) * kMlpMaxBatch * kMlpRowFloats) ==
+            cudaMalloc(&c->mlp_part_dev, sizeof(float) * kMlpPartFloats * c->sm_count) ==
                 cudaSuccess;
   ok = ok && cudaMemset(c->status_dev, 0, 256) == cudaSuccess &&
        cudaMemset(c->slots_dev, 0, kSlotBytes * OMPRT_SLOTS) == cudaSuccess &&
@@ -198,7 +198,7 @@ omprt_status omprt_init(int device, omprt_ctx** out) {
     cudaFree(c->status_dev);
     cudaFree(c->slots_dev);
     cudaFree(c->pool_dev);
-    cudaFree(c->mlp_rows_dev);
+    cudaFree(c->mlp_part_dev);
     cudaGetLastError();
     delete c;
     return OMPRT_ERR_NOMEM;
@@ -213,7 +213,7 @@ omprt_status omprt_finalize(omprt_ctx* c) {
   cudaFree(c->status_dev);
   cudaFree(c->slots_dev);
   cudaFree(c->pool_dev);
-  cudaFree(c->mlp_rows_dev);
+  cudaFree(c->mlp_part_dev);
   delete c;
   return OMPRT_OK;
 }

@@ -16,7 +16,7 @@ struct omprt_ctx {
   uint32_t* status_dev = nullptr;
   unsigned char* slots_dev = nullptr;
   unsigned char* pool_dev = nullptr;
-  float* mlp_rows_dev = nullptr;   // MLP per-sample scratch, kMlpMaxBatch rows
+  float* mlp_part_dev = nullptr;   // MLP partial gradients, one a CTA (one CTA an SM)
   uint32_t stack_bytes = 0;
   uint32_t stage_bytes = 32768;    // per-team shared memory for staged dynamic schedules
   uint32_t stencil_stage_bytes = 0;  // per-CTA shared memory for the staged 2-D stencil windows
@@ -31,9 +31,10 @@ struct omprt_ctx {
   float feat_std[OMPRT_MLP_IN];
 };
 
-// MLP training batch limit and per-sample scratch row (floats).
+// MLP training batch limit, and the floats of one partial gradient (the
+// parameters, the loss, padding to 16 bytes).
 constexpr int kMlpMaxBatch = 16384;
-constexpr int kMlpRowFloats = 272;
+constexpr int kMlpPartFloats = 6032;
 
 struct DeviceGuard {
   int prev = 0;

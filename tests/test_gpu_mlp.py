@@ -114,3 +114,35 @@ def test_choose_config_fallbacks(rt):
     rt.set_cost_model(None)
     f = rt.loop_features(d, False)
     assert f[0] == 16.0 and f[1] == 12.0 and f[3] == 1.0 and f[8] == 0.0
+
+
+# Batches around a CTA's eight samples and around one group of them an SM, and a
+# parameter vector that does not start on 16 bytes, against fp64 autograd.  The
+# bound: at most 16384 terms of magnitude up to the gradient's scale, each within
+# a few fp32 roundings of its value: 2e-6 of the largest entry.
+@pytest.mark.parametrize("B", [1, 7, 8, 9, 1215, 1216, 1217, 2500])
+@pytest.mark.parametrize("off", [0, 1])
+def test_loss_grad_sample_groups(rt, B, off):
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(B)
+    buf = torch.randn(R.MLP_NPARAM + 4, generator=g, device="cuda") * 0.2
+    p = buf[off:off + R.MLP_NPARAM]
+    x = torch.randn(B, 16, generator=g, device="cuda")
+    t = torch.randn(B, 12, generator=g, device="cuda")
+    grad = torch.full((R.MLP_NPARAM + 1,), -7.0, device="cuda")
+    loss = torch.zeros(1, device="cuda")
+    rt.mlp_loss_grad(p, x, t, grad[:R.MLP_NPARAM], loss)
+    q = p.double().requires_grad_(True)
+    w1, b1, w2, b2, w3, b3 = q.split([1024, 64, 4096, 64, 768, 12])
+    h = torch.relu(x.double() @ w1.view(64, 16).T + b1)
+    h = torch.relu(h @ w2.view(64, 64).T + b2)
+    y = h @ w3.view(12, 64).T + b3
+    want = (y - t.double()).square().mean()
+    (dq,) = torch.autograd.grad(want, q)
+    assert float((grad[:-1].double() - dq).abs().max()) <= 2e-6 * float(dq.abs().max())
+    assert abs(float(loss) - float(want)) <= 2e-6 * float(want)
+    assert float(grad[-1]) == -7.0  # nothing written past the parameters
+    out = torch.zeros(B, 12, device="cuda")
+    rt.mlp_forward(p, x, out)
+    assert float((out.double() - y.detach()).abs().max()) <= 2e-6 * float(y.detach().abs().max())
+    assert rt.sync_status() == 0
