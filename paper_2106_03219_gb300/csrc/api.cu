@@ -545,6 +545,12 @@ static omprt_status launch_region_impl(omprt_ctx* c, const omprt_loop_desc* d, i
                                c->status_dev, st);
     if (e != cudaErrorNotSupported) return from_cuda(e);
     cudaGetLastError();
+    // grids the tiles do not take (odd rows, arrays off 16 bytes): strips of
+    // columns (k_stencil_cols.cu)
+    e = launch_stencil2d_cols(d->x, (float*)d->out, (uint64_t)d->nx, (uint64_t)d->ny, (float)d->c0,
+                              (float)d->c1, (unsigned)teams, (unsigned)threads, st);
+    if (e != cudaErrorNotSupported) return from_cuda(e);
+    cudaGetLastError();
   }
   // teams of one warp whose blocks are several rows of one 32-chunk group
   // (m = nx / c < 32): the CTA's warps on adjacent teams, one tensor copy a

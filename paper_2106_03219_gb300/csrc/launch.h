@@ -155,6 +155,12 @@ cudaError_t launch_stencil2d_tiles(const void* in, float* out, uint64_t nx, uint
                                    float c1, unsigned teams, unsigned threads, uint32_t* status,
                                    cudaStream_t st);
 
+// schedule(auto) 2-D stencil by strips of 128 columns a warp, any row length and
+// alignment (k_stencil_cols.cu); cudaErrorNotSupported (nothing launched) for
+// grids beyond its 32-bit counts.
+cudaError_t launch_stencil2d_cols(const void* in, float* out, uint64_t nx, uint64_t ny, float c0,
+                                  float c1, unsigned teams, unsigned threads, cudaStream_t st);
+
 // static(c) 2-D stencil with the team's rows staged through a ring in shared
 // memory (k_stencil_rows.cu): c in [4, 8) and [32, 128], where it beats the
 // plain form; cudaErrorNotSupported (nothing launched) elsewhere.
