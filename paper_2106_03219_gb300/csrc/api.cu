@@ -600,6 +600,15 @@ static omprt_status launch_region_impl(omprt_ctx* c, const omprt_loop_desc* d, i
     if (e != cudaErrorNotSupported) return from_cuda(e);
     cudaGetLastError();
   }
+  // blocks and rows of any length: each lane's next points with the rows above
+  // and below (rules and figures in k_stencil_pieces.cu)
+  if (d->body == OMPRT_BODY_STENCIL2D5 && acc == kAccNone && d->data_type == OMPRT_F32 &&
+      c->stencil_stage_bytes != 0) {
+    e = launch_stencil2d_pieces(ksched, (unsigned)teams, (unsigned)threads, c->max_smem_optin,
+                                c->stage_bytes != 0, st, a);
+    if (e != cudaErrorNotSupported) return from_cuda(e);
+    cudaGetLastError();
+  }
   // dynamic(c) outside the slab form, team blocks of whole rows: the row
   // ring (4096^2 dynamic(256): 0.47 of the copy rate against 0.44 in the
   // streamed ring below)

@@ -161,6 +161,14 @@ cudaError_t launch_stencil2d_tiles(const void* in, float* out, uint64_t nx, uint
 cudaError_t launch_stencil2d_cols(const void* in, float* out, uint64_t nx, uint64_t ny, float c0,
                                   float c1, unsigned teams, unsigned threads, cudaStream_t st);
 
+// static, static(c), dynamic(c) and nonmonotonic dynamic 2-D stencil, team
+// blocks and rows of any length, each lane's next points staged with the rows
+// above and below (k_stencil_pieces.cu); cudaErrorNotSupported (nothing
+// launched) where that form does not apply.
+// row_ring: whether launch_stencil2d_rows may run.
+cudaError_t launch_stencil2d_pieces(int sched, unsigned teams, unsigned threads, int max_smem,
+                                    bool row_ring, cudaStream_t st, const RegionArgs& a);
+
 // static(c) 2-D stencil with the team's rows staged through a ring in shared
 // memory (k_stencil_rows.cu): c in [4, 8) and [32, 128], where it beats the
 // plain form; cudaErrorNotSupported (nothing launched) elsewhere.
