@@ -26,7 +26,11 @@ struct omprt_ctx {
   std::atomic<uint32_t> next_slot{0};
   // learned schedule (host copy of the model)
   bool has_model = false;
-  float model[OMPRT_MLP_NPARAM];
+  // W1, W2, W3 with the outputs of one input side by side (W[in][out]), so that
+  // inference runs over outputs in vector registers; b1, b2, b3 as they are
+  float w1t[OMPRT_MLP_IN * OMPRT_MLP_HID], w2t[OMPRT_MLP_HID * OMPRT_MLP_HID],
+      w3t[OMPRT_MLP_HID * OMPRT_MLP_OUT];
+  float b1[OMPRT_MLP_HID], b2[OMPRT_MLP_HID], b3[OMPRT_MLP_OUT];
   float feat_mean[OMPRT_MLP_IN];
   float feat_std[OMPRT_MLP_IN];
 };

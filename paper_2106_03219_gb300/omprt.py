@@ -146,20 +146,43 @@ def check(status, what="omprt"):
         raise OmprtError(status, what)
 
 
+# Marshalling of a launch.  A small region runs for a few microseconds, so what
+# a call costs here is what a program of small regions waits for: torch is looked
+# up once, the current stream is read without building a torch.cuda.Stream (3.2 us
+# of the call), and pointers go to ctypes as plain integers.  On the GPU host's
+# Arm cores a launch_region takes 3.5 us (7.0 before), a reduce 4.0 (8.4), of
+# them 2.8 in the library and the CUDA launch.
+_torch = None
+_dtype_codes = None
+
+
+def _bind_torch():
+    """Look torch up on first use: the module itself does not need it."""
+    global _torch, _dtype_codes
+    import torch
+    _dtype_codes = {torch.float32: F32, torch.bfloat16: BF16, torch.int32: I32, torch.int64: I64,
+                    torch.int16: BF16, torch.uint16: BF16}
+    _torch = torch
+
+
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
-    import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _torch is None:
+        _bind_torch()
+    if not _torch.cuda.is_initialized():
+        return _torch.cuda.current_stream().cuda_stream
+    return _torch._C._cuda_getCurrentRawStream(_torch._C._cuda_getDevice())
 
 
 def _dtype_code(t):
-    import torch
-    return {torch.float32: F32, torch.bfloat16: BF16, torch.int32: I32, torch.int64: I64,
-            torch.int16: BF16, torch.uint16: BF16}[t.dtype]
+    if _torch is None:
+        _bind_torch()
+    return _dtype_codes[t.dtype]
 
 
 def loop_desc(body, n=None, x=None, y=None, out=None, *, lb=0, ub=None, incr=1, idx_type=I64,
@@ -191,6 +214,7 @@ class Runtime:
         check(lib().omprt_init(int(device), C.byref(ctx)), "omprt_init")
         self.ctx = ctx
         self.device = device
+        self._lib = lib()
 
     def close(self):
         """omprt_finalize: free the context (streams must be synchronised)."""
@@ -241,16 +265,17 @@ class Runtime:
         """omprt_launch_region: run desc's loop under sched / chunk on teams x threads
         (0: defaults); red (ReduceDesc) adds a reduction.  Asynchronous on stream."""
         rd = None if red is None else C.byref(red)
-        check(lib().omprt_launch_region(self.ctx, C.byref(desc), int(sched), int(chunk),
-                                        int(teams), int(threads), rd, _stream(stream)),
-              "omprt_launch_region")
+        st = self._lib.omprt_launch_region(self.ctx, C.byref(desc), int(sched), int(chunk),
+                                           int(teams), int(threads), rd, _stream(stream))
+        if st != OK:
+            check(st, "omprt_launch_region")
 
     def launch_region_dist(self, desc, dist_chunk, sched=SCHED_STATIC, chunk=0, teams=0,
                            threads=0, red=None, stream=None):
         """omprt_launch_region_dist: dist_schedule(static, dist_chunk) at the team
         level, sched / chunk inside each distribute chunk."""
         rd = None if red is None else C.byref(red)
-        check(lib().omprt_launch_region_dist(self.ctx, C.byref(desc), int(dist_chunk), int(sched),
+        check(self._lib.omprt_launch_region_dist(self.ctx, C.byref(desc), int(dist_chunk), int(sched),
                                              int(chunk), int(teams), int(threads), rd,
                                              _stream(stream)), "omprt_launch_region_dist")
 
@@ -260,7 +285,7 @@ class Runtime:
         device tensor of nseg + 1 offsets; result: float64[nseg] (GENERIC_REDUCE)
         or float64[3 * nseg] (GENERIC_DOT_AXPY: v, a, w per segment)."""
         nseg = max(int(seg.numel()) - 1, 0)
-        check(lib().omprt_launch_generic(self.ctx, _ptr(seg), nseg, C.byref(desc), int(program),
+        check(self._lib.omprt_launch_generic(self.ctx, _ptr(seg), nseg, C.byref(desc), int(program),
                                          _ptr(result), int(teams), int(threads),
                                          _stream(stream)), "omprt_launch_generic")
 
@@ -269,9 +294,11 @@ class Runtime:
         """omprt_reduce: reduction(op) over the device tensor data into result
         (float64[1] for fp32 / bf16 data, int64[1] for integers)."""
         dt = _dtype_code(data) if dtype is None else dtype
-        check(lib().omprt_reduce(self.ctx, int(op), int(dt), int(precision), _ptr(data),
-                                 int(data.numel()), _ptr(result), int(teams), int(threads),
-                                 _stream(stream)), "omprt_reduce")
+        st = self._lib.omprt_reduce(self.ctx, int(op), int(dt), int(precision), data.data_ptr(),
+                                    data.numel(), _ptr(result), int(teams), int(threads),
+                                    _stream(stream))
+        if st != OK:
+            check(st, "omprt_reduce")
 
     def static_init_table(self, desc, chunk, teams, threads, table, stream=None):
         """omprt_static_init_table: table (int64 device tensor [G*T][8]) gets every
@@ -325,19 +352,19 @@ class Runtime:
     # -- MLP --------------------------------------------------------------------
     def mlp_forward(self, params, x, y, stream=None):
         """omprt_mlp_forward: y[B][12] = model(x[B][16]) (device tensors)."""
-        check(lib().omprt_mlp_forward(self.ctx, _ptr(params), _ptr(x), int(x.shape[0]), _ptr(y),
+        check(self._lib.omprt_mlp_forward(self.ctx, _ptr(params), _ptr(x), int(x.shape[0]), _ptr(y),
                                       _stream(stream)), "omprt_mlp_forward")
 
     def mlp_loss_grad(self, params, x, target, grad, loss=None, stream=None):
         """omprt_mlp_loss_grad: grad = d loss / d params; loss[1] if given (device tensors)."""
-        check(lib().omprt_mlp_loss_grad(self.ctx, _ptr(params), _ptr(x), _ptr(target),
+        check(self._lib.omprt_mlp_loss_grad(self.ctx, _ptr(params), _ptr(x), _ptr(target),
                                         int(x.shape[0]), _ptr(grad), _ptr(loss),
                                         _stream(stream)), "omprt_mlp_loss_grad")
 
     def mlp_adam(self, params, grad, m, v, t, lr=1e-3, beta1=0.9, beta2=0.999, eps=1e-8,
                  stream=None):
         """omprt_mlp_adam: one bias-corrected Adam step on params (device tensors)."""
-        check(lib().omprt_mlp_adam(self.ctx, _ptr(params), _ptr(grad), _ptr(m), _ptr(v),
+        check(self._lib.omprt_mlp_adam(self.ctx, _ptr(params), _ptr(grad), _ptr(m), _ptr(v),
                                    int(params.numel()), int(t), lr, beta1, beta2, eps,
                                    _stream(stream)), "omprt_mlp_adam")
 
