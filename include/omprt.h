@@ -206,8 +206,8 @@ omprt_status omprt_alloc_shared(omprt_ctx *ctx, size_t bytes_per_team);
  * 512 bytes and the two halos at most a quarter of the pass.  A claim of 32
  * chunks runs in equal passes.  Streaming bodies whose blocks do not all
  * start on a 16-byte boundary, or whose passes do not fit, take the row form
- * where their pieces are long enough (128 bytes under static(c) and
- * dynamic(c), 256 under static): each lane's next 64 or 128 bytes of its piece
+ * where their pieces are long enough (128 bytes under static(c), dynamic(c) and
+ * guided(c), 256 under static): each lane's next 64 or 128 bytes of its piece
  * at a time, in buffers sized from the device's shared memory, whatever
  * `bytes`.  Other launches run the plain form.  The 2-D stencil under
  * static(c) with c in [4, 8) or [32, 128] (fp32, no reduction, nx a multiple of

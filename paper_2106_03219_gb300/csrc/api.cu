@@ -526,7 +526,7 @@ static omprt_status launch_region_impl(omprt_ctx* c, const omprt_loop_desc* d, i
     }
   }
   if (!a.stage_chunks && (ksched == kStatic || ksched == kChunked || ksched == kDynamic ||
-                          ksched == kNonmono)) {
+                          ksched == kGuided || ksched == kNonmono)) {
     const RowPlan rp = row_plan(c, d, sh, n, ksched, (uint64_t)chunk,
                                 (uint32_t)teams, (uint32_t)threads, smem, acc == kAccCompF32);
     if (rp.row_bytes) {

@@ -858,81 +858,104 @@ __device__ __forceinline__ bool run_dist(const Body& b, uint64_t n, uint64_t d, 
 
 // schedule(guided, c) inside the team block [bs, bs + bn): each request takes
 // max(c, ceil(r / 2T)) of the r iterations not yet handed out (never more
-// than r).  Lane 0 of a warp claims the next (up to) 32 such chunks with one
-// compare-and-swap on the team's counter, writing their starts to the warp's
-// row in shared memory as it computes them; every lane then runs the chunk
-// its row entries bound.  The sizes depend only on r, so the partition is the
-// same on every run.
+// than r).  A warp claims the next (up to) 32 such chunks with one
+// compare-and-swap on the team's counter and every lane runs its own of them.
+// The sizes depend only on r, so the partition is the same on every run.
+//
+// The counter lives in team-shared memory: a claim reads it, computes, and
+// swaps, and from global memory the two round trips (and the warps that lost
+// the swap and computed again) bounded whole launches.  Once ceil(r / 2T) <= c
+// every chunk is c, and the 32 starts need no recurrence.  Before that all
+// lanes run the recurrence side by side, in 32-bit arithmetic where the block
+// allows, and each keeps its own step.  Measured, axpy guided(64), n = 2^26,
+// global counter and 64-bit recurrence -> this (with the row form): 608 x 256
+// 235 -> 165 us, 500 x 512 568 -> 204, 333 x 1024 1242 -> 281; n = 2^22, 608 x 256
+// 29.7 -> 13.7.
 __device__ __forceinline__ uint64_t guided_size(uint64_t r, uint64_t c, uint64_t twoT) {
   const uint64_t want = (r + twoT - 1) / twoT;
   const uint64_t s = want > c ? want : c;
   return s < r ? s : r;
 }
-// the same with 2T = 2^sh (a shift instead of a 64-bit division)
-__device__ __forceinline__ uint64_t guided_size_sh(uint64_t r, uint64_t c, uint32_t sh) {
-  const uint64_t want = (r + (1ull << sh) - 1) >> sh;
-  const uint64_t s = want > c ? want : c;
-  return s < r ? s : r;
-}
 
 constexpr uint32_t kGuidedMaxTries = 1u << 20;
-// per warp: the 32 chunk starts of its current guided claim and the claim's end
-static __shared__ unsigned long long rt_guided_row[OMPRT_MAX_THREADS / 32][33];
+static __shared__ unsigned long long rt_guided_next;
 
-// Lane 0 claims the team's next (up to) 32 guided chunks, writing their starts
-// and the claim's end to the warp's row.  Returns false (uniform over the
-// warp) when the block is used up or the bounded retries ran out.  Kept out
-// of line: inlined, its 32-step size loop shaped the register allocation of
-// the streaming loop around it, and guided axpy at n = 2^26 ran at 0.29 /
-// 0.64 / 0.37 of the copy rate for c = 1 / 64 / 256 against 0.48 / 0.84 /
-// 0.84 out of line.
-static __device__ __noinline__ bool guided_claim(unsigned long long* row, uint64_t bn, uint64_t c,
-                                             unsigned long long* ctr, uint32_t* status) {
-  const uint64_t twoT = 2ull * blockDim.x;
-  const bool pow2 = (twoT & (twoT - 1)) == 0;
-  const uint32_t sh = (uint32_t)__ffsll((long long)twoT) - 1;
-  int done = 0;
-  if (lane_id() == 0) {
-    uint32_t tries = 0;
-    for (;;) {
-      const unsigned long long cur = atomicAdd(ctr, 0ull);
-      if (cur >= bn) {
-        done = 1;
-        break;
+// The calling lane's chunk [x, y) of the warp's next claim (x == y: none left
+// for it), or x = ~0 for the whole warp when the block is used up or the
+// bounded retries ran out.  Reached by the whole warp.  Out of line: inlined,
+// its loop shapes the register allocation of the streaming loop around it.
+static __device__ __noinline__ ulonglong2 guided_claim(uint64_t bn, uint64_t c, uint32_t* status) {
+  const uint32_t lane = lane_id(), twoT = 2u * blockDim.x;
+  for (uint32_t tries = 0; tries < kGuidedMaxTries; ++tries) {
+    unsigned long long cur = 0;
+    if (lane == 0) cur = *(volatile unsigned long long*)&rt_guided_next;
+    cur = __shfl_sync(0xffffffffu, cur, 0);
+    if (cur >= bn) return make_ulonglong2(~0ull, 0ull);
+    const uint64_t r = bn - cur;
+    uint64_t lo, hi, next;
+    if (r < (1ull << 58) && (c >= r || (c < (1ull << 40) && r <= c * twoT))) {
+      const uint64_t s = c < r ? c : r;  // every chunk from here on
+      lo = lane * s < r ? lane * s : r;
+      hi = r - lo > s ? lo + s : r;
+      next = 32 * s < r ? 32 * s : r;
+    } else if (r < (1ull << 31)) {
+      const uint32_t r32 = (uint32_t)r, c32 = (uint32_t)c;  // c < r here
+      const bool pow2 = (twoT & (twoT - 1)) == 0;
+      const uint32_t sh = 31 - __clz(twoT);
+      uint32_t p = 0, l = 0, h = 0;
+#pragma unroll 4
+      for (uint32_t k = 0; k < 32; ++k) {
+        const uint32_t left = r32 - p;
+        const uint32_t want = pow2 ? (left + twoT - 1) >> sh : (left + twoT - 1) / twoT;
+        const uint32_t size = min(max(want, c32), left);
+        if (k == lane) {
+          l = p;
+          h = p + size;
+        }
+        p += size;
       }
-      uint64_t pos = cur;
-      for (int k = 0; k < 32; ++k) {
-        row[k] = pos;
-        if (pos < bn) pos += pow2 ? guided_size_sh(bn - pos, c, sh) : guided_size(bn - pos, c, twoT);
+      lo = l;
+      hi = h;
+      next = p;
+    } else {
+      uint64_t p = 0;
+      lo = hi = 0;
+      for (uint32_t k = 0; k < 32; ++k) {
+        const uint64_t size = guided_size(r - p, c, twoT);
+        if (k == lane) {
+          lo = p;
+          hi = p + size;
+        }
+        p += size;
       }
-      row[32] = pos;
-      if (atomicCAS(ctr, cur, (unsigned long long)pos) == cur) break;
-      if (++tries >= kGuidedMaxTries) {  // bounded: give up, report, leave the loop
-        set_status(status, OMPRT_DEV_TIMEOUT);
-        done = 1;
-        break;
-      }
+      next = p;
     }
+    uint32_t won = 0;
+    if (lane == 0) won = atomicCAS(&rt_guided_next, cur, cur + (unsigned long long)next) == cur;
+    if (__shfl_sync(0xffffffffu, won, 0)) return make_ulonglong2(cur + lo, cur + hi);
   }
-  done = __shfl_sync(0xffffffffu, done, 0);
-  __syncwarp();  // the row lane 0 wrote is visible to the warp
-  return !done;
+  if (lane == 0) set_status(status, OMPRT_DEV_TIMEOUT);  // bounded: give up, report
+  return make_ulonglong2(~0ull, 0ull);
+}
+
+// Before the team's first claim; ends in a team barrier.
+__device__ __forceinline__ void guided_start() {
+  if (threadIdx.x == 0) rt_guided_next = 0;
+  team_barrier();
 }
 
 template <class Body, class Acc>
 __device__ __forceinline__ bool run_guided(const Body& b, uint64_t bs, uint64_t bn, uint64_t c,
-                                           unsigned long long* ctr, uint32_t* status,
-                                           Acc& acc) {
-  const uint32_t lane = lane_id();
-  unsigned long long* const row = rt_guided_row[warp_id()];
+                                           uint32_t* status, Acc& acc) {
   bool last = false;
-  while (guided_claim(row, bn, c, ctr, status)) {
-    const uint64_t pos = row[lane], end = row[lane + 1];
-    if (pos < end) {
-      run_range(b, bs + pos, bs + end, acc);
-      if (end == bn) last = true;
+  for (;;) {
+    const ulonglong2 k = guided_claim(bn, c, status);
+    if (k.x == ~0ull) break;
+    if (k.x < k.y) {
+      run_range(b, bs + k.x, bs + k.y, acc);
+      if (k.y == bn) last = true;
     }
-    __syncwarp();  // the row is read before lane 0 writes the next claim's
+    __syncwarp();
   }
   return last;
 }
@@ -1281,10 +1304,8 @@ __global__ void __launch_bounds__(OMPRT_MAX_THREADS) region_kernel(const RegionA
       }
       last = team_last && nch > 0 && (nch - 1) % T == t;
     } else if constexpr (SCHED == kGuided) {
-      unsigned long long* ctr = a.dyn_next + g;
-      last = run_guided(body, bs, bn, a.chunk ? a.chunk : 1, ctr, a.status, acc) && team_last;
-      team_barrier();
-      if (t == 0) *ctr = 0;  // leave the counter at zero for the next launch
+      guided_start();
+      last = run_guided(body, bs, bn, a.chunk ? a.chunk : 1, a.status, acc) && team_last;
     } else if constexpr (SCHED == kNonmono) {
       // nonmonotonic dynamic: per-warp ranges of chunk groups in shared memory
       __shared__ unsigned long long nm_next[OMPRT_MAX_THREADS / 32], nm_end[OMPRT_MAX_THREADS / 32];

@@ -1,7 +1,7 @@
 // The row form: per-thread contiguous pieces moved through shared memory.
 //
-// Under static, static(c), dynamic(c) and nonmonotonic dynamic every thread
-// runs contiguous pieces of the loop.  Read straight from global memory, a
+// Under static, static(c), dynamic(c), nonmonotonic dynamic and guided every
+// thread runs contiguous pieces of the loop.  Read straight from global memory, a
 // warp instruction then touches 32 lines, one per lane, and the launch is
 // bound by L1 wavefronts (ncu of axpy dynamic(256), 608 x 256, n = 2^26: L1
 // 91 % busy, DRAM 52 %, lg_throttle and long scoreboard 170 cycles an issue)
@@ -60,6 +60,18 @@ struct PieceChunks {  // 32 consecutive chunks of c a claim, lane l running base
       h = bn - l > c ? l + c : bn;
     }
     return true;
+  }
+};
+
+struct PieceGuided {  // a warp's guided claims
+  static constexpr bool kAnyWarp = true;
+  uint64_t bn, c;
+  uint32_t* status;
+  __device__ __forceinline__ bool next(uint64_t& l, uint64_t& h) {
+    const ulonglong2 k = guided_claim(bn, c, status);
+    l = k.x;
+    h = k.y;
+    return k.x != ~0ull;
   }
 };
 
@@ -258,7 +270,8 @@ __device__ __forceinline__ void run_rows(const Body& b, const RegionArgs& a, uin
 template <class Body, int SCHED>
 constexpr bool rows_for() {
   return Stageable<Body>::value && !StageHalo<Body>::value &&
-         (SCHED == kStatic || SCHED == kChunked || SCHED == kDynamic || SCHED == kNonmono);
+         (SCHED == kStatic || SCHED == kChunked || SCHED == kDynamic || SCHED == kGuided ||
+          SCHED == kNonmono);
 }
 
 // The row form's kernel: the region kernel's levels and epilogue around
@@ -286,7 +299,7 @@ __global__ void __launch_bounds__(OMPRT_MAX_THREADS) rows_kernel(const RegionArg
       run_rows<64>(body, a, bs, pieces, acc);
   };
   const uint64_t c = a.chunk;
-  const uint64_t nch = SCHED != kStatic && bn ? (bn - 1) / c + 1 : 0;
+  const uint64_t nch = SCHED != kStatic && SCHED != kGuided && bn ? (bn - 1) / c + 1 : 0;
   if constexpr (SCHED == kStatic) {
     uint64_t s, cnt;
     split_even(bn, T, t, s, cnt);
@@ -299,6 +312,9 @@ __global__ void __launch_bounds__(OMPRT_MAX_THREADS) rows_kernel(const RegionArg
     run(PieceChunks<ClaimDynamic>{ClaimDynamic{ctr}, nch, c, bn});
     team_barrier();
     if (t == 0) *ctr = 0;  // leave the counter at zero for the next launch
+  } else if constexpr (SCHED == kGuided) {
+    guided_start();  // and rt_row_slots is set
+    run(PieceGuided{bn, c, a.status});
   } else {
     __shared__ unsigned long long nm_next[OMPRT_MAX_THREADS / 32], nm_end[OMPRT_MAX_THREADS / 32];
     const uint32_t w = warp_id(), W = T / 32;

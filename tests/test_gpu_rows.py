@@ -1,5 +1,5 @@
-"""GPU parity: the row form of static, static(c), dynamic(c) and nonmonotonic
-dynamic (each lane's next row of its piece staged through shared memory).
+"""GPU parity: the row form of static, static(c), dynamic(c), nonmonotonic
+dynamic and guided (each lane's next row of its piece staged through shared memory).
 
 Sizes put piece ends at every place of a 16-byte unit and of a row, blocks of
 too few chunks beside long ones, teams of every buffer shape (two and more
@@ -18,7 +18,7 @@ pytestmark = pytest.mark.gpu
 
 SCHEDS = [(R.SCHED_STATIC, 0), (R.SCHED_STATIC_CHUNKED, 32), (R.SCHED_STATIC_CHUNKED, 61),
           (R.SCHED_STATIC_CHUNKED, 1000), (R.SCHED_DYNAMIC, 64), (R.SCHED_DYNAMIC, 257),
-          (R.SCHED_NONMONOTONIC, 96)]
+          (R.SCHED_NONMONOTONIC, 96), (R.SCHED_GUIDED, 32), (R.SCHED_GUIDED, 301)]
 SHAPES = [(1, 32), (3, 128), (5, 256), (2, 512), (3, 1024)]
 NS = [40_961, 300_006, (1 << 20) + 3]
 
@@ -52,7 +52,8 @@ def test_axpy_rows_bit_exact(rt, sched, chunk, G, T):
 
 
 @pytest.mark.parametrize("sched,chunk", [(R.SCHED_STATIC, 0), (R.SCHED_STATIC_CHUNKED, 61),
-                                         (R.SCHED_DYNAMIC, 514), (R.SCHED_NONMONOTONIC, 96)])
+                                         (R.SCHED_DYNAMIC, 514), (R.SCHED_NONMONOTONIC, 96),
+                                         (R.SCHED_GUIDED, 64)])
 @pytest.mark.parametrize("G,T", SHAPES)
 def test_value_reductions_rows(rt, sched, chunk, G, T):
     import torch
