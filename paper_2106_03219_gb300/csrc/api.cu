@@ -147,6 +147,27 @@ static omprt_status pick_acc(const omprt_loop_desc* d, const omprt_reduce_desc* 
   return OMPRT_ERR_INVALID;
 }
 
+int32_t auto_teams(int32_t body, int32_t data_type, uintptr_t pointers, uint64_t n, int32_t teams,
+                   int32_t threads) {
+  uint64_t vec;  // iterations a 32-byte vector
+  switch (body) {
+    case OMPRT_BODY_AXPY:
+    case OMPRT_BODY_DOT:
+    case OMPRT_BODY_STENCIL1D3:
+      vec = 8;
+      break;
+    case OMPRT_BODY_NONE:
+      vec = data_type == OMPRT_BF16 ? 16 : data_type == OMPRT_I64 ? 4 : 8;
+      break;
+    default: return teams;  // map record reports every team; the 2-D grid maps otherwise
+  }
+  // without the vector path, and for what no whole vector holds, one iteration
+  // a thread
+  const uint64_t items = (pointers & 31) ? n : n / vec;
+  const uint64_t useful = items ? (items - 1) / (uint64_t)threads + 1 : 1;
+  return useful < (uint64_t)teams ? (int32_t)useful : teams;
+}
+
 static omprt_status from_cuda(cudaError_t e) {
   if (e == cudaSuccess) return OMPRT_OK;
   if (e == cudaErrorNotSupported) return OMPRT_ERR_UNSUPPORTED;
@@ -469,6 +490,12 @@ static omprt_status launch_region_impl(omprt_ctx* c, const omprt_loop_desc* d, i
   const bool counters = ksched == kDynamic || ksched == kGuided;
   if ((acc != kAccNone || counters) && teams > OMPRT_MAX_RED_TEAMS) return OMPRT_ERR_INVALID;
 
+  if (ksched == kAuto)
+    teams = auto_teams(d->body, d->data_type,
+                       (uintptr_t)d->x | (d->body == OMPRT_BODY_STENCIL1D3 ? (uintptr_t)d->out
+                                          : d->body == OMPRT_BODY_NONE     ? 0
+                                                                           : (uintptr_t)d->y),
+                       n, teams, threads);
   DeviceGuard guard(c->device);
   rt::OverlapScope overlap(c->launch_overlap, (size_t)c->smem_per_sm);
   RegionArgs a;

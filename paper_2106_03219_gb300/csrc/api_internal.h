@@ -56,6 +56,16 @@ ScratchSlot ctx_next_slot(omprt_ctx* ctx);
 
 omprt_status loop_trip_count(const omprt_loop_desc* d, uint64_t* n, int64_t* wide_lb);
 
+// Teams of a schedule(auto) launch of a one-dimensional body that get an
+// iteration: the mapping hands 32-byte vectors to threads in order, grid-stride,
+// so with fewer vectors than threads the teams after the last vector run
+// nothing.  They are not launched: the others' iterations are the same, and a
+// reduction has fewer partials to wait for (10,007 int64 values on 304 x 512: 5
+// teams instead of 304, 4.2 -> 4.0 us; one team 4.0 -> 1.9; without allocation,
+// 4096 teams by default, 36 -> 8.3).
+int32_t auto_teams(int32_t body, int32_t data_type, uintptr_t pointers, uint64_t n, int32_t teams,
+                   int32_t threads);
+
 struct LearnedConfig {
   int32_t sched;
   int64_t chunk;

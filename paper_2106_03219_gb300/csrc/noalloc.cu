@@ -82,14 +82,16 @@ extern "C" omprt_status omprt_reduce_noalloc(int32_t op, int32_t dtype, int32_t 
     case OMPRT_OP_MIN: acc = integer ? kAccMinI64 : kAccMinF32; break;
     default: return OMPRT_ERR_INVALID;
   }
+  teams = auto_teams(OMPRT_BODY_NONE, dtype, (uintptr_t)data, (uint64_t)n, teams, threads);
   unsigned char* scratch;
   omprt_status s = scratch_for_current_device(&scratch);
   if (s) return s;
   cudaStream_t st = (cudaStream_t)stream;
   // A completed launch leaves its ticket at 0 (atomicInc(ticket, G - 1) wraps
   // on the last team); this clear, in stream order, only repairs a ticket (and
-  // status word) left behind by a launch that did not run to the end.
-  if (cudaMemsetAsync(scratch, 0, 8, st) != cudaSuccess) {
+  // status word) left behind by a launch that did not run to the end.  One
+  // team takes no ticket.
+  if (teams > 1 && cudaMemsetAsync(scratch, 0, 8, st) != cudaSuccess) {
     cudaGetLastError();
     return OMPRT_ERR_CUDA;
   }

@@ -1004,6 +1004,20 @@ __device__ inline void reduce_epilogue(const Acc& acc, const RegionArgs& a) {
   if (scratch == nullptr) return;                  // flagged OMPRT_DEV_STACK_NOMEM
   const P v = team_reduce<Acc>(acc.part(), (P*)scratch);
   constexpr bool kComp = std::is_same<P, float2>::value;
+  if (gridDim.x == 1) {  // nothing to wait for: the one partial is the result
+    if (threadIdx.x == 0) {
+      if constexpr (kComp) {
+        if (a.prec == OMPRT_PREC_COMP_F64)
+          write_result(a.result, __dadd_rn(0.0, __dadd_rn((double)v.x, (double)v.y)));
+        else
+          write_result(a.result, Acc::merge(Acc::identity(), v));
+      } else {
+        write_result(a.result, Acc::merge(Acc::identity(), v));
+      }
+    }
+    team_free(scratch, 32 * 16, a.status);
+    return;
+  }
   if (threadIdx.x == 0) {
     unsigned char* slot = a.partials + 16ull * blockIdx.x;
     if constexpr (kComp) {
@@ -1016,12 +1030,14 @@ __device__ inline void reduce_epilogue(const Acc& acc, const RegionArgs& a) {
       store_part(slot, v);
     }
     flush();  // the partial is visible device-wide before the ticket
-    const uint32_t tk = atomic_inc(a.ticket, gridDim.x - 1);
+    // the bare hardware inc: the flushes on both sides are this function's, and
+    // only the team that draws the last ticket needs the second
+    const uint32_t tk = atomicInc(a.ticket, gridDim.x - 1);
     rt_bcast_flag = (tk == gridDim.x - 1);
+    if (tk == gridDim.x - 1) flush();  // every team's partial is visible after it
   }
   team_barrier();
   if (rt_bcast_flag) {
-    flush();
     if constexpr (kComp) {
       if (a.prec == OMPRT_PREC_COMP_F64)
         combine_partials<CombF64, double>(a, scratch);
