@@ -234,8 +234,11 @@ omprt_status omprt_set_stage_bytes(omprt_ctx *ctx, int64_t bytes_per_team);
  * claimed from the team's counter in shared memory, 32 per warp, lane l
  * running chunk base + l; a thread's claims increase.  The form applies when
  * nx is a multiple of 4, n < 2^32, both pointers are 16-byte aligned,
- * thread_limit <= 512 and the ring holds one team's rows with room to spare;
- * other launches run the forms of omprt_set_stage_bytes.  bytes is rounded
+ * thread_limit <= 512 and the ring holds one team's rows with room to spare.
+ * Launches whose blocks or rows line up with nothing (any nx, static, static(c),
+ * dynamic(c), nonmonotonic) hold a team's whole block and one row on each side
+ * where that fits `bytes`, else stage each thread's next points with the rows
+ * above and below; other launches run the forms of omprt_set_stage_bytes.  bytes is rounded
  * down to 16; 0 turns this form off, and with it the slab, band and column-ring
  * forms of omprt_set_stencil_slab_shape and the row ring of
  * dynamic(c) (those size their buffers from the device's shared memory);

@@ -627,10 +627,16 @@ static omprt_status launch_region_impl(omprt_ctx* c, const omprt_loop_desc* d, i
     if (e != cudaErrorNotSupported) return from_cuda(e);
     cudaGetLastError();
   }
-  // blocks and rows of any length: each lane's next points with the rows above
-  // and below (rules and figures in k_stencil_pieces.cu)
+  // blocks and rows of any length: the whole block and a grid row on each side in
+  // shared memory where they fit, else each lane's next points with the rows
+  // above and below (rules and figures in k_stencil_window.cu, k_stencil_pieces.cu)
   if (d->body == OMPRT_BODY_STENCIL2D5 && acc == kAccNone && d->data_type == OMPRT_F32 &&
       c->stencil_stage_bytes != 0) {
+    int budget = c->max_smem_optin - 2048;
+    if ((int64_t)c->stencil_stage_bytes < budget) budget = (int)c->stencil_stage_bytes;
+    e = launch_stencil2d_window(ksched, (unsigned)teams, (unsigned)threads, budget, st, a);
+    if (e != cudaErrorNotSupported) return from_cuda(e);
+    cudaGetLastError();
     e = launch_stencil2d_pieces(ksched, (unsigned)teams, (unsigned)threads, c->max_smem_optin,
                                 c->stage_bytes != 0, st, a);
     if (e != cudaErrorNotSupported) return from_cuda(e);

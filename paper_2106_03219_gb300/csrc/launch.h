@@ -169,6 +169,12 @@ cudaError_t launch_stencil2d_cols(const void* in, float* out, uint64_t nx, uint6
 cudaError_t launch_stencil2d_pieces(int sched, unsigned teams, unsigned threads, int max_smem,
                                     bool row_ring, cudaStream_t st, const RegionArgs& a);
 
+// the same schedules, a team's whole block and a grid row on each side in shared
+// memory, at most `budget` bytes (k_stencil_window.cu); cudaErrorNotSupported
+// (nothing launched) where that form does not apply.
+cudaError_t launch_stencil2d_window(int sched, unsigned teams, unsigned threads, int budget,
+                                    cudaStream_t st, const RegionArgs& a);
+
 // static(c) 2-D stencil with the team's rows staged through a ring in shared
 // memory (k_stencil_rows.cu): c in [4, 8) and [32, 128], where it beats the
 // plain form; cudaErrorNotSupported (nothing launched) elsewhere.

@@ -1,5 +1,6 @@
-"""GPU parity: the 2-D stencil on grids and team blocks of any length: lanes'
-pieces staged with the rows above and below (static, static(c), dynamic(c),
+"""GPU parity: the 2-D stencil on grids and team blocks of any length: a team's
+whole block in shared memory, or (the budget too small for it) lanes' pieces
+staged with the rows above and below (static, static(c), dynamic(c),
 nonmonotonic), and strips of columns (auto on odd grids).
 
 Grids put rows at every place of a 16-byte unit, rows shorter than a staged
@@ -18,7 +19,7 @@ pytestmark = pytest.mark.gpu
 
 GRIDS = [(1, 4099), (4099, 1), (2051, 2), (1400, 3), (900, 5), (301, 33), (130, 127), (129, 514),
          (67, 1001), (255, 256), (40, 4095), (33, 4100)]
-SCHEDS = [(R.SCHED_STATIC, 0), (R.SCHED_STATIC_CHUNKED, 32), (R.SCHED_STATIC_CHUNKED, 61),
+SCHEDS = [(R.SCHED_STATIC, 0), (R.SCHED_STATIC_CHUNKED, 9), (R.SCHED_STATIC_CHUNKED, 32), (R.SCHED_STATIC_CHUNKED, 61),
           (R.SCHED_STATIC_CHUNKED, 300), (R.SCHED_DYNAMIC, 33), (R.SCHED_DYNAMIC, 64),
           (R.SCHED_NONMONOTONIC, 100)]
 
@@ -38,10 +39,18 @@ def _check(rt, ny, nx, sched, chunk, G, T, off=0):
 
 
 @pytest.mark.parametrize("sched,chunk", SCHEDS)
-@pytest.mark.parametrize("G,T", [(1, 32), (3, 96), (2, 256), (1, 512)])
-def test_pieces_bit_exact(rt, sched, chunk, G, T):
-    for ny, nx in GRIDS:
-        _check(rt, ny, nx, sched, chunk, G, T)
+@pytest.mark.parametrize("G,T", [(1, 32), (3, 96), (2, 256), (1, 512), (4, 1024)])
+@pytest.mark.parametrize("budget", [16, 226 * 1024])  # pieces; windows where they fit
+def test_pieces_and_windows_bit_exact(rt, sched, chunk, G, T, budget):
+    rt.set_stencil_stage_bytes(budget)
+    try:
+        for ny, nx in GRIDS:
+            _check(rt, ny, nx, sched, chunk, G, T)
+            if nx == 514 or nx == 1001:  # small blocks: short windows, empty threads
+                _check(rt, ny, nx, sched, chunk, 40 * G, T)
+            _check(rt, ny, nx, sched, chunk, 2 * G, T, 4)  # off 32 bytes, on 16
+    finally:
+        rt.set_stencil_stage_bytes(226 * 1024)
     assert rt.sync_status() == 0
 
 
