@@ -218,7 +218,8 @@ static cudaError_t launch_window_odd(bool odd, unsigned teams, unsigned threads,
 // Returns cudaErrorNotSupported, launching nothing, where this form does not
 // apply (a window beyond `budget` bytes) or loses to the others: pieces under
 // 8 points (16 under static), and blocks under 1024 points on grids of whole
-// 16-byte units (700 x 600, static(64), 608 x 256: 6.0 us in the others, 6.7 here).
+// 16-byte units (700 x 600, static(64), 608 x 256: 6.0 us in the others, 6.7 here)
+// or with chunks under 32 (293 x 1034, static(8), 1142 x 256: 7.3, 8.8 here).
 cudaError_t launch_stencil2d_window(int sched, unsigned teams, unsigned threads, int budget,
                                     cudaStream_t st, const RegionArgs& a) {
   const bool whole = sched == kStatic, odd = a.nx % 4 != 0;
@@ -227,8 +228,9 @@ cudaError_t launch_stencil2d_window(int sched, unsigned teams, unsigned threads,
       ((uintptr_t)a.out & 31))
     return cudaErrorNotSupported;
   const uint64_t block = (a.n - 1) / teams + 1;
-  if ((whole ? block / threads : a.chunk) < (whole ? 16u : 8u) || block > (1ull << 24) ||
-      (!odd && block < 1024))
+  const uint64_t piece = whole ? block / threads : a.chunk;
+  if (piece < (whole ? 16u : 8u) || block > (1ull << 24) ||
+      (block < 1024 && (!odd || piece < 32)))
     return cudaErrorNotSupported;
   WindowArgs P;
   P.r = a;
