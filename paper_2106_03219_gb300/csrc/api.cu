@@ -541,7 +541,7 @@ static omprt_status launch_region_impl(omprt_ctx* c, const omprt_loop_desc* d, i
   // not all do, streaming bodies take the row form instead (axpy static(64)
   // at n = 2^26, 900 x 128: 227 -> 139 us)
   const bool aligned = n % (uint64_t)teams == 0 && n / (uint64_t)teams * sh.elem % 16 == 0;
-  if (stage_c && (aligned || sh.halo)) {
+  if (stage_c && (aligned || d->body == OMPRT_BODY_STENCIL2D5)) {
     const StagePlan sp = stage_plan(c, sh, stage_c, (uint32_t)threads, smem,
                                     acc != kAccNone);
     if (sp.chunks) {
@@ -675,6 +675,14 @@ static omprt_status launch_region_impl(omprt_ctx* c, const omprt_loop_desc* d, i
     e = launch_stencil2d_rows(d->x, (float*)d->out, (uint64_t)d->nx, (uint64_t)d->ny,
                               (uint64_t)chunk, (float)d->c0, (float)d->c1, (unsigned)teams,
                               (unsigned)threads, c->max_smem_optin, c->status_dev, st);
+    if (e != cudaErrorNotSupported) return from_cuda(e);
+    cudaGetLastError();
+  }
+  // the 1-D stencil outside the staged form: each lane's next points staged
+  if (d->body == OMPRT_BODY_STENCIL1D3 && acc == kAccNone && !a.stage_chunks &&
+      c->stage_bytes != 0) {
+    e = launch_stencil1d_pieces(ksched, (unsigned)teams, (unsigned)threads, c->max_smem_optin, st,
+                                a);
     if (e != cudaErrorNotSupported) return from_cuda(e);
     cudaGetLastError();
   }

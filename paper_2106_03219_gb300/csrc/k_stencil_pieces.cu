@@ -219,17 +219,132 @@ __device__ __forceinline__ void run_stencil_pieces(const BodyStencil2D& b,
   }
 }
 
+// 1-D 3-point stencil: the same slabs without rows above and below.  A lane's
+// row: the unit left of it, its NU units, the unit right of it, one of padding.
+constexpr uint32_t kLineNu = 8;
+constexpr uint32_t kLineStage = 32 * 16 * (kLineNu + 4);
+template <class Pieces>
+__device__ __forceinline__ void run_line_pieces(const BodyStencil1D& b, uint64_t bs,
+                                                Pieces& pieces) {
+  constexpr uint32_t NU = kLineNu, RE = 4 * NU, kLane = (NU + 3) * 16;
+  const uint32_t lane = lane_id();
+  const uint64_t n = b.n;
+  unsigned char* st = nullptr;  // this warp's rows, from its first claim on
+  uint64_t pos = 0, end = 0;
+  const uint32_t cu = lane % NU, cr = lane / NU, k4 = 4 * cu;
+  for (;;) {
+    while (!__any_sync(0xffffffffu, pos < end)) {
+      if (!pieces.next(pos, end)) return;
+      pos += bs;
+      end += bs;
+    }
+    if (!st) {
+      uint32_t slot = warp_id();
+      if constexpr (Pieces::kAnyWarp) {
+        if (lane == 0) slot = atomicAdd(&rt_row_slots, 1u);
+        slot = __shfl_sync(0xffffffffu, slot, 0);
+      }
+      st = rt_dyn_smem + (size_t)slot * kLineStage;
+    }
+    uint4* const rec = (uint4*)(st + 32 * kLane);
+    const uint64_t row = pos / RE * RE;
+    uint32_t j0 = 0, j1 = 0;
+    const uint32_t ce = n - row < RE + 8 ? (uint32_t)(n - row) : RE + 8;  // its elements in x
+    if (pos < end) {
+      j0 = (uint32_t)(pos - row);
+      j1 = end - row < RE ? (uint32_t)(end - row) : RE;
+      pos = row + j1;
+    }
+    const char* const src = (const char*)(b.in + row);
+    rec[lane] = make_uint4((uint32_t)(uintptr_t)src, (uint32_t)((uintptr_t)src >> 32),
+                           j0 | j1 << 8, ce);
+    if (j0 < j1) {  // the units beside the row, each fetched by its lane
+      const uint32_t mine = smem_addr(st) + lane * kLane;
+      cp_async_if(j0 == 0 && row > 0, mine, src - 16, 16);
+      cp_async_if(j1 == RE && ce > RE, mine + (NU + 1) * 16, src + RE * 4,
+                  min(16u, (ce - RE) * 4));
+    }
+    __syncwarp();
+#pragma unroll
+    for (uint32_t q = 0; q < NU; ++q) {
+      const uint32_t l = q * (32 / NU) + cr;
+      const uint4 m = rec[l];
+      const uint32_t i0 = m.z & 255u, i1 = m.z >> 8;
+      cp_async_if(i0 < i1 && k4 <= i1 && k4 + 4 >= i0 && k4 < m.w,
+                  smem_addr(st) + l * kLane + cu * 16 + 16,
+                  (const char*)(((uint64_t)m.y << 32) | m.x) + cu * 16, min(16u, (m.w - k4) * 4));
+    }
+    cp_async_commit();
+    cp_async_wait(0);
+    __syncwarp();  // every lane's copies have landed
+    if (j0 < j1) {
+      float4* const mine = (float4*)(st + lane * kLane);
+      const bool inner = row >= 1 && row + RE < n;  // no end point in the row
+      float w = mine[0].w;
+      float4 cc = mine[1];
+#pragma unroll
+      for (uint32_t u = 0; u < NU; ++u) {
+        const float4 nx = mine[u + 2];
+        float4 o = make_float4(b.point(w, cc.x, cc.y), b.point(cc.x, cc.y, cc.z),
+                               b.point(cc.y, cc.z, cc.w), b.point(cc.z, cc.w, nx.x));
+        if (!inner) {
+          const uint64_t i = row + 4 * u;
+          if (i == 0 || i + 1 == n) o.x = cc.x;
+          if (i + 2 == n) o.y = cc.y;
+          if (i + 3 == n) o.z = cc.z;
+          if (i + 4 == n) o.w = cc.w;
+        }
+        mine[u + 1] = o;
+        w = cc.w;
+        cc = nx;
+      }
+      auto part = [&](uint32_t u) {  // a unit with another piece's points beside this lane's
+        const float4 o = mine[u + 1];
+        const float v[4] = {o.x, o.y, o.z, o.w};
+#pragma unroll
+        for (uint32_t q = 0; q < 4; ++q)
+          if (4 * u + q >= j0 && 4 * u + q < j1) b.out[row + 4 * u + q] = v[q];
+      };
+      if (j0 % 4) part(j0 / 4);
+      if (j1 % 4 && (j0 % 4 == 0 || j0 / 4 != j1 / 4)) part(j1 / 4);
+    }
+    __syncwarp();
+#pragma unroll
+    for (uint32_t h = 0; h < NU; h += 4) {
+      uint4 m[4], v[4];
+#pragma unroll
+      for (uint32_t q = 0; q < 4; ++q) {
+        const uint32_t l = (h + q) * (32 / NU) + cr;
+        m[q] = rec[l];
+        v[q] = *(const uint4*)(st + l * kLane + 16 + cu * 16);
+      }
+#pragma unroll
+      for (uint32_t q = 0; q < 4; ++q)
+        st16_if(k4 >= (m[q].z & 255u) && k4 + 4 <= m[q].z >> 8,
+                (char*)b.out + ((const char*)(((uint64_t)m[q].y << 32) | m[q].x) - (const char*)b.in) +
+                    cu * 16,
+                v[q]);
+    }
+    __syncwarp();  // the rows have been read: the next slab may land
+  }
+}
+
 constexpr unsigned kPieceThreads = 512;  // largest team: 128 registers a thread
-template <int SCHED, uint32_t NU>
-__global__ void __launch_bounds__(kPieceThreads) stencil_pieces_kernel(const StencilPieceArgs P) {
+template <int SCHED, uint32_t NU>  // NU 0: the 1-D stencil
+__global__ void __launch_bounds__(NU ? kPieceThreads : 1024)
+    stencil_pieces_kernel(const StencilPieceArgs P) {
   enter_region_grid();
   const RegionArgs& a = P.r;
   const uint32_t g = blockIdx.x, t = threadIdx.x, T = blockDim.x;
-  const BodyStencil2D body(a);
   if (t == 0) rt_row_slots = 0;
   uint64_t bs, bn;
   split_even(a.n, gridDim.x, g, bs, bn);
-  auto run = [&](auto pieces) { run_stencil_pieces<NU>(body, P, bs, pieces); };
+  auto run = [&](auto pieces) {
+    if constexpr (NU == 0)
+      run_line_pieces(BodyStencil1D(a), bs, pieces);
+    else
+      run_stencil_pieces<NU>(BodyStencil2D(a), P, bs, pieces);
+  };
   const uint64_t c = a.chunk;
   const uint64_t nch = SCHED != kStatic && bn ? (bn - 1) / c + 1 : 0;
   if constexpr (SCHED == kStatic) {
@@ -245,7 +360,7 @@ __global__ void __launch_bounds__(kPieceThreads) stencil_pieces_kernel(const Ste
     team_barrier();
     if (t == 0) *ctr = 0;  // leave the counter at zero for the next launch
   } else {
-    __shared__ unsigned long long nm_next[kPieceThreads / 32], nm_end[kPieceThreads / 32];
+    __shared__ unsigned long long nm_next[32], nm_end[32];
     const uint32_t w = warp_id(), W = T / 32;
     if (lane_id() == 0) {
       uint64_t s0, cnt;
@@ -318,6 +433,38 @@ cudaError_t launch_stencil2d_pieces(int sched, unsigned teams, unsigned threads,
     case kChunked: return launch_pieces_nu<kChunked>(nu, teams, threads, smem, st, P);
     case kDynamic: return launch_pieces_nu<kDynamic>(nu, teams, threads, smem, st, P);
     default: return launch_pieces_nu<kNonmono>(nu, teams, threads, smem, st, P);
+  }
+}
+
+// The 1-D stencil: chunks of 32 points on in blocks of 32 chunks (n = 2^26, 608 x
+// 256: static(64) 210 -> 129 us, dynamic(256) 151 -> 143, 500 x 512 187 -> 144; n =
+// 2^24 static(32) 78 -> 42, dynamic(64) 58 -> 36; n = 2^22 dynamic(256), 27 chunks a
+// block: 15.6 -> 16.1), and under static pieces of 64 to 256 points and from 1024
+// on (608 x 256: 107 points 42 -> 38 us, 431 points 123 -> 138; 148 x 128, 3542
+// points 222 -> 181).  Returns cudaErrorNotSupported, launching nothing, elsewhere.
+cudaError_t launch_stencil1d_pieces(int sched, unsigned teams, unsigned threads, int max_smem,
+                                    cudaStream_t st, const RegionArgs& a) {
+  const bool whole = sched == kStatic;
+  if ((sched != kStatic && sched != kChunked && sched != kDynamic && sched != kNonmono) ||
+      a.n == 0 || (((uintptr_t)a.x | (uintptr_t)a.out) & 15))
+    return cudaErrorNotSupported;
+  const uint64_t block = (a.n - 1) / teams + 1, piece = whole ? block / threads : a.chunk;
+  if (piece < (whole ? 64u : 32u) || (whole && piece > 256 && piece < 1024))
+    return cudaErrorNotSupported;
+  uint32_t warps = threads / 32;  // that can be busy at once
+  if (!whole) {
+    const uint64_t chunks = (block - 1) / a.chunk + 1;
+    if (chunks < 32) return cudaErrorNotSupported;
+    if ((chunks + 31) / 32 < warps) warps = (uint32_t)((chunks + 31) / 32);
+  }
+  const size_t smem = (size_t)warps * kLineStage;
+  if ((int64_t)smem > (int64_t)max_smem - 1024) return cudaErrorNotSupported;
+  const StencilPieceArgs P = {a, 0u, 0u};
+  switch (sched) {
+    case kStatic: return launch_pieces<kStatic, 0>(teams, threads, smem, st, P);
+    case kChunked: return launch_pieces<kChunked, 0>(teams, threads, smem, st, P);
+    case kDynamic: return launch_pieces<kDynamic, 0>(teams, threads, smem, st, P);
+    default: return launch_pieces<kNonmono, 0>(teams, threads, smem, st, P);
   }
 }
 

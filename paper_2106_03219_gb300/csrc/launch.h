@@ -169,6 +169,10 @@ cudaError_t launch_stencil2d_cols(const void* in, float* out, uint64_t nx, uint6
 cudaError_t launch_stencil2d_pieces(int sched, unsigned teams, unsigned threads, int max_smem,
                                     bool row_ring, cudaStream_t st, const RegionArgs& a);
 
+// The 1-D stencil the same way (without rows above and below).
+cudaError_t launch_stencil1d_pieces(int sched, unsigned teams, unsigned threads, int max_smem,
+                                    cudaStream_t st, const RegionArgs& a);
+
 // the same schedules, a team's whole block and a grid row on each side in shared
 // memory, at most `budget` bytes (k_stencil_window.cu); cudaErrorNotSupported
 // (nothing launched) where that form does not apply.

@@ -76,3 +76,20 @@ def test_runtime_team_counts_and_budget_off(rt):
     finally:
         rt.set_stencil_stage_bytes(226 * 1024)
     assert rt.sync_status() == 0
+
+
+@pytest.mark.parametrize("sched,chunk", SCHEDS)
+@pytest.mark.parametrize("G,T", [(1, 32), (3, 96), (2, 256), (3, 1024)])
+def test_stencil1d_pieces_bit_exact(rt, sched, chunk, G, T):
+    import torch
+    for n in (1, 2, 33, 4100, 40_961, 300_006, (1 << 20) + 3):
+        for off in (0, 4):
+            a = inputs.f32_uniform01(n + 8, 4)
+            out = torch.full((n + 8,), -7.0, device="cuda")
+            rt.launch_region(R.loop_desc(R.BODY_STENCIL1D3, n=n, x=dev(a)[off:off + n],
+                                         out=out[off:off + n]), sched, chunk, G, T)
+            got = host(out)
+            want = O.stencil1d3(np.ascontiguousarray(a[off:off + n]))
+            assert np.array_equal(bits32(got[off:off + n]), bits32(want)), (n, off)
+            assert (got[:off] == -7.0).all() and (got[off + n:] == -7.0).all()
+    assert rt.sync_status() == 0
