@@ -77,7 +77,8 @@ typedef enum {
     OMPRT_SCHED_DYNAMIC = 2,        /* chunks of c claimed at run time from a
                                        per-team counter in global memory */
     OMPRT_SCHED_AUTO = 3,           /* mapping left to the runtime: grid-stride
-                                       over 32-byte vectors */
+                                       over 32-byte vectors (teams that would get
+                                       no iteration are not launched) */
     OMPRT_SCHED_LEARNED = 4,        /* schedule, chunk and teams chosen by the
                                        context's cost model (see
                                        omprt_set_cost_model), else the heuristic */

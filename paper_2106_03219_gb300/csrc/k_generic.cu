@@ -533,7 +533,11 @@ extern "C" omprt_status omprt_launch_generic(omprt_ctx* c, const int64_t* seg_de
   while (a.tile_log2 > 10 && room < 3 * (8 << a.tile_log2)) --a.tile_log2;
   const int64_t fit = std::min<int64_t>(room > 0 ? room / (8 << a.tile_log2) : 0, kTilesMax);
   a.tiles = (uint32_t)fit;
-  if (fit < 2 || threads > (int)kTiledThreads || (((uintptr_t)d->x | (uintptr_t)d->y) & 15)) {
+  // Tiles are loaded segments ahead: not where a segment's y is another's x
+  // (arrays that overlap without being the same).
+  const uintptr_t xa = (uintptr_t)d->x, ya = (uintptr_t)d->y;
+  const bool overlap_xy = xa != ya && (xa < ya ? ya - xa : xa - ya) < n * 4;
+  if (fit < 2 || threads > (int)kTiledThreads || ((xa | ya) & 15) || overlap_xy) {
     static const size_t static_bytes = static_smem_of(generic_kernel);
     if (smem_optin(generic_kernel, a.stack_bytes, static_bytes) != cudaSuccess) {
       cudaGetLastError();
