@@ -390,9 +390,11 @@ static cudaError_t launch_pieces_nu(uint32_t nu, unsigned teams, unsigned thread
                  : launch_pieces<SCHED, 4>(teams, threads, smem, st, P);
 }
 
-// Returns cudaErrorNotSupported, launching nothing, where this form does not
-// apply or loses to the others (4096^2 and 2048^2, plain or ring forms against
-// this one, G x T teams x threads):
+// Tried after the block window (k_stencil_window.cu), which takes most of these
+// launches where a team's block fits shared memory.  Returns
+// cudaErrorNotSupported, launching nothing, where this form does not apply or
+// loses to the others (4096^2 and 2048^2, plain or ring forms against this one,
+// G x T teams x threads):
 //   - pieces of 32 points on; teams of up to 512 threads;
 //   - odd grids (nx no multiple of 4): always (3001 x 2503, 608 x 256: static
 //     98 -> 37 us, static(32) 166 -> 45, static(128) 166 -> 31, static(500) 178
