@@ -13,10 +13,11 @@
 // reads two rows more than it writes.
 //
 // Before, odd grids ran point by point (five loads and a 64-bit row split a
-// point: 62 % issue active).  3001 x 2503, 608 x 256: 24.8 -> 14.8 us (0.61 of the
-// copy rate), 4095^2: 54.7 -> 29.7 (0.68).  128 columns and four rows fetched at
-// a time, without a standing pipeline: 18.2 and 34.1.  What bounds it: pieces of
-// 25 rows start and end cold, and the shuffles and selects.
+// point: 62 % issue active).  3001 x 2503, 608 x 256: 24.8 -> 13.8 us (0.65 of the
+// copy rate), 4095^2: 54.7 -> 28.7 (0.70).  128 columns and four rows fetched at
+// a time, without a standing pipeline: 18.2 and 34.1; every column and row of
+// every strip tested: 14.8 and 29.7 (72 % issue active).  What bounds it: issue
+// (shuffles, selects), and pieces of 25 rows that start and end cold.
 #include "launch_common.cuh"
 
 namespace rt {
@@ -35,72 +36,95 @@ struct ColsArgs {
 constexpr uint32_t kStrip = 64;  // columns a warp
 constexpr uint32_t kAhead = 5;   // rows in flight
 
-__global__ void __launch_bounds__(1024) stencil2d_cols_kernel(const ColsArgs A) {
-  enter_region_grid();
+// Rows [r0, r1) of the strip at col0.  kFull: the strip and the columns beside it
+// are inner columns (all but the first and last strips), so no column is tested.
+template <bool kFull>
+__device__ __forceinline__ void walk_strip(const ColsArgs& A, uint64_t col0, uint32_t r0,
+                                           uint32_t r1) {
   const uint32_t lane = lane_id();
   const uint64_t nx = A.nx;
+  const uint32_t rl = r1 < A.ny ? r1 : A.ny - 1;  // the last row it reads
+  // this lane's columns inside the grid, whether they are inner ones, and
+  // the column it fetches beside the strip (lane 0 the one before it, lane
+  // 31 the one after)
+  const uint64_t left = nx - col0;
+  const bool ok0 = kFull || lane < left, ok1 = kFull || lane + 32 < left;
+  const bool in0 = kFull || ((lane || col0) && lane + 1 < left);
+  const bool in1 = kFull || lane + 33 < left;
+  const bool side = kFull ? lane == 0 || lane == 31
+                          : (lane == 0 ? col0 > 0 : lane == 31 && kStrip < left);
+  const int64_t beside = lane == 0 ? -1 : 33;
+  const float* src = A.in + (uint64_t)r0 * nx + col0 + lane;
+  float* out = A.out + (uint64_t)r0 * nx + col0 + lane;
+  float u0 = 0.f, u1 = 0.f, d0[kAhead], d1[kAhead], de[kAhead];
+  if (r0 > 0) {
+    u0 = ok0 ? ld_nc(src - nx) : 0.f;
+    u1 = ok1 ? ld_nc(src - nx + 32) : 0.f;
+  }
+  float c0 = ok0 ? ld_nc(src) : 0.f, c1 = ok1 ? ld_nc(src + 32) : 0.f;
+  float edge = side ? ld_nc(src + beside) : 0.f;
+  uint32_t q = r0;  // the last row on its way; past rl the last row comes again
+  auto fetch = [&](uint32_t k) {
+    if (q < rl) {
+      src += nx;
+      ++q;
+    }
+    d0[k] = ok0 ? ld_nc(src) : 0.f;
+    d1[k] = ok1 ? ld_nc(src + 32) : 0.f;
+    de[k] = side ? ld_nc(src + beside) : 0.f;
+  };
+#pragma unroll
+  for (uint32_t k = 0; k < kAhead; ++k) fetch(k);
+  auto row = [&](uint32_t k, bool inner) {
+    // lane 0 gets lane 31's, lane 31 lane 0's
+    const float w0 = __shfl_sync(0xffffffffu, c0, (lane + 31) & 31),
+                w1 = __shfl_sync(0xffffffffu, c1, (lane + 31) & 31),
+                e0 = __shfl_sync(0xffffffffu, c0, (lane + 1) & 31),
+                e1 = __shfl_sync(0xffffffffu, c1, (lane + 1) & 31);
+    const float wa = lane == 0 ? edge : w0, ea = lane == 31 ? e1 : e0;
+    const float wb = lane == 0 ? w0 : w1, eb = lane == 31 ? edge : e1;
+    const float a = __fmaf_rn(A.c1, __fadd_rn(__fadd_rn(u0, d0[k]), __fadd_rn(ea, wa)),
+                              __fmul_rn(A.c0, c0));
+    const float b = __fmaf_rn(A.c1, __fadd_rn(__fadd_rn(u1, d1[k]), __fadd_rn(eb, wb)),
+                              __fmul_rn(A.c0, c1));
+    if (ok0) out[0] = inner && in0 ? a : c0;
+    if (ok1) out[32] = inner && in1 ? b : c1;
+    out += nx;
+    u0 = c0;
+    u1 = c1;
+    c0 = d0[k];
+    c1 = d1[k];
+    edge = de[k];
+    fetch(k);
+  };
+  uint32_t r = r0;
+  for (; r + kAhead <= r1; r += kAhead) {
+    const bool mid = r > 0 && r + kAhead < A.ny;  // no boundary row among them
+    if (mid) {
+#pragma unroll
+      for (uint32_t k = 0; k < kAhead; ++k) row(k, true);
+    } else {
+#pragma unroll
+      for (uint32_t k = 0; k < kAhead; ++k) row(k, r + k > 0 && r + k + 1 < A.ny);
+    }
+  }
+#pragma unroll
+  for (uint32_t k = 0; k < kAhead; ++k)
+    if (r + k < r1) row(k, r + k > 0 && r + k + 1 < A.ny);
+}
+
+__global__ void __launch_bounds__(1024) stencil2d_cols_kernel(const ColsArgs A) {
+  enter_region_grid();
   const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x / 32);
   for (uint64_t p = (uint64_t)blockIdx.x * (blockDim.x / 32) + warp_id(); p < A.pieces;
        p += warps) {
     const uint64_t col0 = p % A.strips * kStrip;
     const uint32_t r0 = (uint32_t)(p / A.strips) * A.rows;
     const uint32_t r1 = A.ny - r0 < A.rows ? A.ny : r0 + A.rows;
-    const uint32_t rl = r1 < A.ny ? r1 : A.ny - 1;  // the last row it reads
-    // this lane's columns inside the grid, whether they are inner ones, and
-    // the column it fetches beside the strip (lane 0 the one before it, lane
-    // 31 the one after)
-    const uint64_t left = nx - col0;
-    const bool ok0 = lane < left, ok1 = lane + 32 < left;
-    const bool in0 = (lane || col0) && lane + 1 < left, in1 = lane + 33 < left;
-    const bool side = lane == 0 ? col0 > 0 : lane == 31 && kStrip < left;
-    const int64_t beside = lane == 0 ? -1 : 33;
-    const float* src = A.in + (uint64_t)r0 * nx + col0 + lane;
-    float* out = A.out + (uint64_t)r0 * nx + col0 + lane;
-    float u0 = 0.f, u1 = 0.f, d0[kAhead], d1[kAhead], de[kAhead];
-    if (r0 > 0) {
-      u0 = ok0 ? ld_nc(src - nx) : 0.f;
-      u1 = ok1 ? ld_nc(src - nx + 32) : 0.f;
-    }
-    float c0 = ok0 ? ld_nc(src) : 0.f, c1 = ok1 ? ld_nc(src + 32) : 0.f;
-    float edge = side ? ld_nc(src + beside) : 0.f;
-    uint32_t q = r0;  // the last row on its way
-    auto fetch = [&](uint32_t k) {
-      ++q;
-      src += nx;
-      const bool in = q <= rl;
-      d0[k] = in && ok0 ? ld_nc(src) : 0.f;
-      d1[k] = in && ok1 ? ld_nc(src + 32) : 0.f;
-      de[k] = in && side ? ld_nc(src + beside) : 0.f;
-    };
-#pragma unroll
-    for (uint32_t k = 0; k < kAhead; ++k) fetch(k);
-    for (uint32_t r = r0; r < r1; r += kAhead) {
-#pragma unroll
-      for (uint32_t k = 0; k < kAhead; ++k) {
-        if (r + k >= r1) break;
-        const bool inner = r + k > 0 && r + k + 1 < A.ny;
-        // lane 0 gets lane 31's, lane 31 lane 0's
-        const float w0 = __shfl_sync(0xffffffffu, c0, (lane + 31) & 31),
-                    w1 = __shfl_sync(0xffffffffu, c1, (lane + 31) & 31),
-                    e0 = __shfl_sync(0xffffffffu, c0, (lane + 1) & 31),
-                    e1 = __shfl_sync(0xffffffffu, c1, (lane + 1) & 31);
-        const float wa = lane == 0 ? edge : w0, ea = lane == 31 ? e1 : e0;
-        const float wb = lane == 0 ? w0 : w1, eb = lane == 31 ? edge : e1;
-        const float a = __fmaf_rn(A.c1, __fadd_rn(__fadd_rn(u0, d0[k]), __fadd_rn(ea, wa)),
-                                  __fmul_rn(A.c0, c0));
-        const float b = __fmaf_rn(A.c1, __fadd_rn(__fadd_rn(u1, d1[k]), __fadd_rn(eb, wb)),
-                                  __fmul_rn(A.c0, c1));
-        if (ok0) out[0] = inner && in0 ? a : c0;
-        if (ok1) out[32] = inner && in1 ? b : c1;
-        out += nx;
-        u0 = c0;
-        u1 = c1;
-        c0 = d0[k];
-        c1 = d1[k];
-        edge = de[k];
-        fetch(k);
-      }
-    }
+    if (col0 > 0 && A.nx - col0 > kStrip)
+      walk_strip<true>(A, col0, r0, r1);
+    else
+      walk_strip<false>(A, col0, r0, r1);
   }
 }
 
