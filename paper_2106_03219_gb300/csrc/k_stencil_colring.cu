@@ -312,7 +312,7 @@ cudaError_t launch_stencil2d_colring(const void* in, float* out, uint64_t nx, ui
           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorNotSupported;
   const size_t smem = (size_t)NB * a.slab + 1024;
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = smem_optin(kern, smem, fa.sharedSizeBytes);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, (int)(32 * K + 32), smem);

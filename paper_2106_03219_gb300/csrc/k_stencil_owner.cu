@@ -459,7 +459,11 @@ cudaError_t launch_stencil2d_owner(const void* in, float* out, uint64_t nx, uint
   auto* kern = sched == kStatic    ? stencil2d_owner_kernel<kStatic>
                : sched == kChunked ? stencil2d_owner_kernel<kChunked>
                                    : stencil2d_owner_kernel<kDynamic>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static const size_t static_bytes[3] = {static_smem_of(stencil2d_owner_kernel<kStatic>),
+                                         static_smem_of(stencil2d_owner_kernel<kChunked>),
+                                         static_smem_of(stencil2d_owner_kernel<kDynamic>)};
+  cudaError_t e = smem_optin(
+      kern, smem, static_bytes[sched == kStatic ? 0 : sched == kChunked ? 1 : 2]);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, (int)(K * threads + 32), smem);

@@ -344,7 +344,7 @@ cudaError_t launch_stencil2d_rowring(const void* in, float* out, uint64_t nx, ui
   a.slots = (uint32_t)S;
   a.pitch = (uint32_t)pitch;
   const size_t smem = (size_t)(S * pitch * 4 + 128);
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = smem_optin(kern, smem, fa.sharedSizeBytes);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, (int)(K * threads + 32), smem);

@@ -350,7 +350,7 @@ cudaError_t launch_stencil2d_slabs(const void* in, float* out, uint64_t nx, uint
   uint64_t K = W / wpt;
   if (K < 1) return cudaErrorNotSupported;
   const size_t smem = (size_t)(K * wpt * NB * a.slab + 1024);
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = smem_optin(kern, smem, fa.sharedSizeBytes);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, (int)(K * threads), smem);

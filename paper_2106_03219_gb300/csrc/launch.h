@@ -12,6 +12,13 @@ namespace rt {
 // A launch gets 48 KB of shared memory, static and dynamic together, without
 // the kernel's opt-in; beyond that the opt-in must cover the dynamic part.
 // The kernel's static part is looked up once per kernel by the caller.
+//
+// The opt-in belongs to the kernel on its device, and all host threads share
+// it.  Every launch therefore sets the same value, all that the device gives
+// beside the static part, and none ever lowers it: set to the size at hand, a
+// smaller launch of the same kernel on another thread could lower it between
+// this thread's opt-in and its launch, which the driver would then refuse.
+// Set anew each time, it also holds after a device reset.
 template <class K>
 inline size_t static_smem_of(K kern) {
   cudaFuncAttributes fa;
@@ -24,7 +31,15 @@ inline size_t static_smem_of(K kern) {
 template <class K>
 inline cudaError_t smem_optin(K kern, size_t dyn, size_t static_bytes) {
   if (dyn + static_bytes <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+  int dev = 0, most = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  // a size beyond the device's limit is passed on for CUDA to refuse
+  const size_t all = (size_t)most > static_bytes ? (size_t)most - static_bytes : 0;
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)(dyn > all ? dyn : all));
 }
 
 // Launch overlap, per host thread: whether executor launches may overlap
