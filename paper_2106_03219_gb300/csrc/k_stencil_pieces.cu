@@ -12,6 +12,7 @@
 // fetched one unit wider and shifted in registers.  Every lane computes its
 // own points, four at a time, and the results leave line by line.
 #include "launch_common.cuh"
+#include "piece_spans.h"
 
 namespace rt {
 
@@ -32,12 +33,12 @@ __device__ __forceinline__ float4 shift4(const float4& a, const float4& b, uint3
   return s & 1 ? make_float4(h.y, h.z, h.w, l) : h;
 }
 
-__device__ __forceinline__ void cp_async_if(bool p, uint32_t dst, const char* src,
-                                            uint32_t bytes) {
+// the first `bytes` of a unit, the rest of it zero; none if bytes is 0
+__device__ __forceinline__ void cp_async_bytes(uint32_t dst, const char* src, uint32_t bytes) {
   asm volatile(
-      "{ .reg .pred q; setp.ne.u32 q, %2, 0; @q cp.async.cg.shared.global [%0], [%1], 16, %3; }" ::
+      "{ .reg .pred q; setp.ne.u32 q, %2, 0; @q cp.async.cg.shared.global [%0], [%1], 16, %2; }" ::
           "r"(dst),
-      "l"(src), "r"((uint32_t)p), "r"(bytes)
+      "l"(src), "r"(bytes)
       : "memory");
 }
 
@@ -47,7 +48,8 @@ __device__ __forceinline__ void cp_async_if(bool p, uint32_t dst, const char* sr
 // of units: the lanes of an access phase hit distinct banks).
 //
 // A lane's record: the row's address, its own points [j0, j1) of it, and how
-// far into the three spans the grid reaches (all in elements, one byte each).
+// far into the three spans the grid reaches (all in elements, one byte each;
+// piece_spans.h).
 template <uint32_t NU, class Pieces>
 __device__ __forceinline__ void run_stencil_pieces(const BodyStencil2D& b,
                                                    const StencilPieceArgs& P, uint64_t bs,
@@ -81,13 +83,7 @@ __device__ __forceinline__ void run_stencil_pieces(const BodyStencil2D& b,
     {
       const uint64_t row = pos / RE * RE;
       uint32_t j0 = 0, j1 = 0;
-      // the spans' elements inside the grid: the row's [0, ce), above [nb, ..),
-      // below [0, se), counted up to RE + 8
-      constexpr uint32_t kTop = RE + 8;
-      const uint32_t ce = n - row < kTop ? (uint32_t)(n - row) : kTop;
-      const uint32_t nb = row >= up ? 0u : up - row < kTop ? (uint32_t)(up - row) : kTop;
-      const uint64_t sb = row + down;
-      const uint32_t se = sb >= n ? 0u : n - sb < kTop ? (uint32_t)(n - sb) : kTop;
+      const PieceSpans sp = piece_spans<RE>(row, n, up, down);
       if (pos < end) {
         j0 = (uint32_t)(pos - row);
         j1 = end - row < RE ? (uint32_t)(end - row) : RE;
@@ -95,16 +91,16 @@ __device__ __forceinline__ void run_stencil_pieces(const BodyStencil2D& b,
       }
       const char* const src = (const char*)(b.in + row);
       rec[lane] = make_uint4((uint32_t)(uintptr_t)src, (uint32_t)((uintptr_t)src >> 32),
-                             j0 | j1 << 8, ce | nb << 8 | se << 16);
+                             j0 | j1 << 8, sp.ce | sp.ab << 8 | sp.be << 16 | sp.ae << 24);
       if (j0 < j1) {  // the units beyond the row's NU, each fetched by its lane
         const uint32_t mine = smem_addr(st) + lane * kLane;
-        cp_async_if(j0 == 0 && row > 0, mine, src - 16, 16);
-        cp_async_if(j1 == RE && ce > RE, mine + (NU + 1) * 16, src + RE * 4,
-                    min(16u, (ce - RE) * 4));
+        cp_async_bytes(mine, src - 16, j0 == 0 && row > 0 ? 16 : 0);
+        cp_async_bytes(mine + (NU + 1) * 16, src + RE * 4, centre_bytes(RE, j0, j1, sp.ce));
         if (sn | ss) {
-          cp_async_if(j1 + sn > RE && nb <= RE, mine + kN + NU * 16, src + RE * 4 - up * 4, 16);
-          cp_async_if(j1 + ss > RE && se > RE, mine + kSo + NU * 16, src + RE * 4 + down * 4,
-                      min(16u, (se - RE) * 4));
+          cp_async_bytes(mine + kN + NU * 16, src + RE * 4 - up * 4,
+                         above_bytes(RE, j0, j1, sn, sp.ab, sp.ae));
+          cp_async_bytes(mine + kSo + NU * 16, src + RE * 4 + down * 4,
+                         below_bytes(RE, j0, j1, ss, sp.be));
         }
       }
       __syncwarp();
@@ -114,14 +110,13 @@ __device__ __forceinline__ void run_stencil_pieces(const BodyStencil2D& b,
         const uint4 m = rec[l];
         const char* const p = (const char*)(((uint64_t)m.y << 32) | m.x) + cu * 16;
         const uint32_t dst = smem_addr(st) + l * kLane + cu * 16;
-        const uint32_t i0 = m.z & 255u, i1 = m.z >> 8, mc = m.w & 255u, mb = m.w >> 8 & 255u,
-                       me = m.w >> 16;
-        const bool some = i0 < i1;
-        cp_async_if(some && k4 <= i1 && k4 + 4 >= i0 && k4 < mc, dst + 16, p,
-                    min(16u, (mc - k4) * 4));
-        cp_async_if(some && k4 < i1 + sn && k4 + 4 > i0 + sn && k4 >= mb, dst + kN, p - up * 4, 16);
-        cp_async_if(some && k4 < i1 + ss && k4 + 4 > i0 + ss && k4 < me, dst + kSo, p + down * 4,
-                    min(16u, (me - k4) * 4));
+        const uint32_t i0 = m.z & 255u, i1 = m.z >> 8;
+        if (i0 < i1) {
+          cp_async_bytes(dst + 16, p, centre_bytes(k4, i0, i1, m.w & 255u));
+          cp_async_bytes(dst + kN, p - up * 4,
+                         above_bytes(k4, i0, i1, sn, m.w >> 8 & 255u, m.w >> 24));
+          cp_async_bytes(dst + kSo, p + down * 4, below_bytes(k4, i0, i1, ss, m.w >> 16 & 255u));
+        }
       }
       cp_async_commit();
     }
@@ -260,9 +255,8 @@ __device__ __forceinline__ void run_line_pieces(const BodyStencil1D& b, uint64_t
                            j0 | j1 << 8, ce);
     if (j0 < j1) {  // the units beside the row, each fetched by its lane
       const uint32_t mine = smem_addr(st) + lane * kLane;
-      cp_async_if(j0 == 0 && row > 0, mine, src - 16, 16);
-      cp_async_if(j1 == RE && ce > RE, mine + (NU + 1) * 16, src + RE * 4,
-                  min(16u, (ce - RE) * 4));
+      cp_async_bytes(mine, src - 16, j0 == 0 && row > 0 ? 16 : 0);
+      cp_async_bytes(mine + (NU + 1) * 16, src + RE * 4, centre_bytes(RE, j0, j1, ce));
     }
     __syncwarp();
 #pragma unroll
@@ -270,9 +264,10 @@ __device__ __forceinline__ void run_line_pieces(const BodyStencil1D& b, uint64_t
       const uint32_t l = q * (32 / NU) + cr;
       const uint4 m = rec[l];
       const uint32_t i0 = m.z & 255u, i1 = m.z >> 8;
-      cp_async_if(i0 < i1 && k4 <= i1 && k4 + 4 >= i0 && k4 < m.w,
-                  smem_addr(st) + l * kLane + cu * 16 + 16,
-                  (const char*)(((uint64_t)m.y << 32) | m.x) + cu * 16, min(16u, (m.w - k4) * 4));
+      if (i0 < i1)
+        cp_async_bytes(smem_addr(st) + l * kLane + cu * 16 + 16,
+                       (const char*)(((uint64_t)m.y << 32) | m.x) + cu * 16,
+                       centre_bytes(k4, i0, i1, m.w));
     }
     cp_async_commit();
     cp_async_wait(0);

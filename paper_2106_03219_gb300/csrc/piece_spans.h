@@ -1,0 +1,57 @@
+// Which bytes of the grid a lane of the 2-D stencil's piece form fetches
+// (k_stencil_pieces.cu): index arithmetic alone, plain C++, so that it can be
+// enumerated on the host.
+//
+// A lane's row is the grid's elements [row, row + RE), row a multiple of RE, of
+// which [j0, j1) are its own.  Three spans are fetched in 16-byte units: the
+// centre at row, the one above at row - up and the one below at row + down, up
+// and down being nx rounded up and down to multiples of 4 (up = nx + sn, down = nx -
+// ss).  Unit k4 of a span starts k4 elements into it, k4 = 0, 4, .. RE; where a span
+// leaves the grid, nothing is fetched before its first element or after its last.
+#pragma once
+
+#include <cstdint>
+
+#ifdef __CUDACC__
+#define RT_HD __host__ __device__ __forceinline__
+#else
+#define RT_HD inline
+#endif
+
+namespace rt {
+
+// How far into each span the grid reaches, in elements, at most RE + 8 (so that
+// a byte holds each): the centre's [0, ce), above [ab, ae), below [0, be).
+struct PieceSpans {
+  uint32_t ce, ab, ae, be;
+};
+template <uint32_t RE>
+RT_HD PieceSpans piece_spans(uint64_t row, uint64_t n, uint64_t up, uint64_t down) {
+  constexpr uint32_t kTop = RE + 8;
+  const uint64_t b = row + down, a = n + up - row;  // row <= n
+  PieceSpans s;
+  s.ce = n - row < kTop ? (uint32_t)(n - row) : kTop;
+  s.ab = row >= up ? 0u : up - row < kTop ? (uint32_t)(up - row) : kTop;
+  s.ae = a < kTop ? (uint32_t)a : kTop;
+  s.be = b >= n ? 0u : n - b < kTop ? (uint32_t)(n - b) : kTop;
+  return s;
+}
+
+// Bytes of a unit inside the first `end` elements of its span.
+RT_HD uint32_t unit_bytes(uint32_t k4, uint32_t end) {
+  return k4 >= end ? 0u : end - k4 < 4 ? (end - k4) * 4 : 16u;
+}
+// Bytes to fetch of unit k4: 0 where none of the lane's points [j0, j1), j0 < j1,
+// reads it.  The centre's also holds the points' neighbours west and east.
+RT_HD uint32_t centre_bytes(uint32_t k4, uint32_t j0, uint32_t j1, uint32_t ce) {
+  return k4 <= j1 && k4 + 4 >= j0 ? unit_bytes(k4, ce) : 0u;
+}
+RT_HD uint32_t above_bytes(uint32_t k4, uint32_t j0, uint32_t j1, uint32_t sn, uint32_t ab,
+                           uint32_t ae) {
+  return k4 < j1 + sn && k4 + 4 > j0 + sn && k4 >= ab ? unit_bytes(k4, ae) : 0u;
+}
+RT_HD uint32_t below_bytes(uint32_t k4, uint32_t j0, uint32_t j1, uint32_t ss, uint32_t be) {
+  return k4 < j1 + ss && k4 + 4 > j0 + ss ? unit_bytes(k4, be) : 0u;
+}
+
+}  // namespace rt
