@@ -105,7 +105,10 @@ __global__ void __launch_bounds__(kThreads) mlp_kernel(const float* __restrict__
   float g2[4][4] = {}, g1[4] = {}, g3[4] = {}, gb = 0.f;
   for (int b0 = blockIdx.x * kS; b0 < B; b0 += gridDim.x * kS) {
     const int ns = B - b0 < kS ? B - b0 : kS;
-    // samples beyond the batch run on zeros and add nothing
+    // Samples beyond the batch run on zeros.  For training their activations are
+    // zeros too, so that they add nothing: what the weights make of an input of
+    // zeros may be beyond fp32's range where no sample of the batch is.
+    const bool real0 = !kTrain || s0 < ns, real1 = !kTrain || s0 + 1 < ns;
     if (t < kS * kIn) S.x[t / kIn][t % kIn] = t < ns * kIn ? X[(size_t)b0 * kIn + t] : 0.f;
     if (kTrain && t >= 128 && t < 128 + kS * kOut) {
       const int q = t - 128;
@@ -120,7 +123,7 @@ __global__ void __launch_bounds__(kThreads) mlp_kernel(const float* __restrict__
       a0 = fma4(w, ld4(&S.x[s0][k]), a0);
       a1 = fma4(w, ld4(&S.x[s0 + 1][k]), a1);
     }
-    const float h1a = fmaxf(a0, 0.f), h1b = fmaxf(a1, 0.f);
+    const float h1a = real0 ? fmaxf(a0, 0.f) : 0.f, h1b = real1 ? fmaxf(a1, 0.f) : 0.f;
     S.h1[s0][u] = h1a;
     S.h1[s0 + 1][u] = h1b;
     __syncthreads();
@@ -132,7 +135,7 @@ __global__ void __launch_bounds__(kThreads) mlp_kernel(const float* __restrict__
       a0 = fma4(w, ld4(&S.h1[s0][k]), a0);
       a1 = fma4(w, ld4(&S.h1[s0 + 1][k]), a1);
     }
-    const float h2a = fmaxf(a0, 0.f), h2b = fmaxf(a1, 0.f);
+    const float h2a = real0 ? fmaxf(a0, 0.f) : 0.f, h2b = real1 ? fmaxf(a1, 0.f) : 0.f;
     S.h2[s0][u] = h2a;
     S.h2[s0 + 1][u] = h2b;
     __syncthreads();

@@ -146,3 +146,36 @@ def test_loss_grad_sample_groups(rt, B, off):
     rt.mlp_forward(p, x, out)
     assert float((out.double() - y.detach()).abs().max()) <= 2e-6 * float(y.detach().abs().max())
     assert rt.sync_status() == 0
+
+
+@pytest.mark.parametrize("B", [1, 3, 8, 13, 255])
+def test_padding_adds_nothing(rt, B):
+    """A batch that is no whole number of sample groups, and weights under which
+    an input of zeros overflows where the batch's own samples do not: unit 0 of
+    layer 1 is off for every sample (x[0] = 1, 2 - 10 < 0) but 2 for zeros, and
+    layer 2 takes it times 3e38.  The samples that fill a group must add nothing, so
+    gradients and loss are those of the batch (2e-6 as above)."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(B)
+    p = torch.randn(R.MLP_NPARAM, generator=g, device="cuda") * 0.2
+    w1, b1, w2, b2, w3, b3 = p.split([1024, 64, 4096, 64, 768, 12])  # views of p
+    w1[:16] = 0.0
+    w1[0], b1[0] = -10.0, 2.0
+    w2[::64] = 0.0  # only unit 0 of layer 2 reads unit 0 of layer 1
+    w2[:64] = 0.0
+    w2[0], b2[0] = 3e38, -1.0
+    x = torch.randn(B, 16, generator=g, device="cuda")
+    x[:, 0] = 1.0
+    t = torch.randn(B, 12, generator=g, device="cuda")
+    grad, loss = torch.zeros(R.MLP_NPARAM, device="cuda"), torch.zeros(1, device="cuda")
+    rt.mlp_loss_grad(p, x, t, grad, loss)
+    q = p.double().requires_grad_(True)
+    w1, b1, w2, b2, w3, b3 = q.split([1024, 64, 4096, 64, 768, 12])
+    h = torch.relu(x.double() @ w1.view(64, 16).T + b1)
+    h = torch.relu(h @ w2.view(64, 64).T + b2)
+    want = (h @ w3.view(12, 64).T + b3 - t.double()).square().mean()
+    (dq,) = torch.autograd.grad(want, q)
+    assert bool(torch.isfinite(grad).all())
+    assert float((grad.double() - dq).abs().max()) <= 2e-6 * float(dq.abs().max())
+    assert abs(float(loss) - float(want.detach())) <= 2e-6 * float(want.detach())
+    assert rt.sync_status() == 0
