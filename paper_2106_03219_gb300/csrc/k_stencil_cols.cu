@@ -19,6 +19,7 @@
 // every strip tested: 14.8 and 29.7 (72 % issue active).  What bounds it: issue
 // (shuffles, selects), and pieces of 25 rows that start and end cold.
 #include "launch_common.cuh"
+#include "plan.h"
 
 namespace rt {
 
@@ -33,7 +34,6 @@ struct ColsArgs {
   uint64_t pieces;
 };
 
-constexpr uint32_t kStrip = 64;  // columns a warp
 constexpr uint32_t kAhead = 5;   // rows in flight
 
 // Rows [r0, r1) of the strip at col0.  kFull: the strip and the columns beside it
@@ -128,15 +128,12 @@ __global__ void __launch_bounds__(1024) stencil2d_cols_kernel(const ColsArgs A) 
   }
 }
 
-// Returns cudaErrorNotSupported, launching nothing, for grids whose strip
-// pieces do not count in 32 bits, and for those of fewer than two points a
-// thread, which the region kernel finishes in one round of loads (301 x 300, 608 x
-// 256: 2.0 us there, 2.5 here; 1001^2, 1000 x 128: 5.2, 3.5 here).
+// Returns cudaErrorNotSupported, launching nothing, where the rule (plan.h) leaves
+// the grid to the region kernel.
 cudaError_t launch_stencil2d_cols(const void* in, float* out, uint64_t nx, uint64_t ny, float c0,
                                   float c1, unsigned teams, unsigned threads, cudaStream_t st) {
+  if (!cols_applies(nx, ny, teams, threads)) return cudaErrorNotSupported;
   const uint64_t strips = (nx + kStrip - 1) / kStrip;
-  if (strips >= (1ull << 31) || ny >= (1ull << 31) || nx * ny < 2ull * teams * threads)
-    return cudaErrorNotSupported;
   ColsArgs a;
   a.in = (const float*)in;
   a.out = out;

@@ -170,9 +170,9 @@ cudaError_t launch_stencil2d_tiles(const void* in, float* out, uint64_t nx, uint
                                    float c1, unsigned teams, unsigned threads, uint32_t* status,
                                    cudaStream_t st);
 
-// schedule(auto) 2-D stencil by strips of 128 columns a warp, any row length and
-// alignment (k_stencil_cols.cu); cudaErrorNotSupported (nothing launched) for
-// grids beyond its 32-bit counts.
+// schedule(auto) 2-D stencil by strips of 64 columns a warp, any row length and
+// alignment (k_stencil_cols.cu); cudaErrorNotSupported (nothing launched) where
+// cols_applies (plan.h) leaves the grid to the region kernel.
 cudaError_t launch_stencil2d_cols(const void* in, float* out, uint64_t nx, uint64_t ny, float c0,
                                   float c1, unsigned teams, unsigned threads, cudaStream_t st);
 
