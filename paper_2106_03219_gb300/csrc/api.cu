@@ -8,6 +8,7 @@
 #include <new>
 
 #include "api_internal.h"
+#include "plan.h"
 
 using namespace rt;
 
@@ -282,13 +283,8 @@ omprt_status omprt_set_stencil_stage_bytes(omprt_ctx* c, int64_t bytes) {
 
 }  // extern "C"
 
-// Arrays a body moves per iteration and their element size, for the staged
-// form of schedules (0 arrays: the body is not staged); halo: elements its
-// input window reaches beyond a pass on each side (the stencils).
-struct StageShape {
-  uint32_t arrays, elem;
-  uint64_t halo;
-};
+// What the plan needs of a body: the arrays it moves per iteration and their
+// element size (0 arrays: the body is not staged).
 static StageShape stage_shape(const omprt_loop_desc* d, uint64_t n) {
   switch (d->body) {
     case OMPRT_BODY_AXPY:
@@ -308,130 +304,6 @@ static StageShape stage_shape(const omprt_loop_desc* d, uint64_t n) {
     default:
       return {0u, 0u, 0};
   }
-}
-
-// Staged pass size for a dynamic(c) / static(c) / static launch: the largest
-// P <= 32 chunks whose buffers (every warp: P chunks of every array) fit the
-// context's per-team staging bytes, or 0 for the plain form.  Measured on
-// GB300 (n = 2^26): chunks below 256 bytes are already coalesced in the plain
-// form and lose to the per-pass overhead (static(8) axpy 0.94 staged against
-// 1.02 plain); without a reduction staging wins from P >= 16 (dynamic(256)
-// 0.97 against 0.64, static(64) 1.02 against 0.97) and loses below
-// (dynamic(1024): P <= 8); with a (compensated) reduction the per-element
-// work needs many warps per SM, and staging wins only with all 32 lanes busy
-// on chunks of at most 512 bytes over all arrays (dot dynamic(64) +16%, sum
-// +9%; dynamic(256) loses).
-struct StagePlan {
-  uint32_t chunks;      // P; 0: the plain form
-  uint32_t warp_bytes;  // shared memory per warp
-};
-static StagePlan stage_plan(const omprt_ctx* c, const StageShape& sh, uint64_t chunk,
-                            uint32_t threads, size_t smem_base, bool reduction) {
-  const StagePlan none = {0u, 0u};
-  if (!sh.arrays || c->stage_bytes == 0) return none;
-  const uint64_t cb = chunk * sh.elem;
-  if (cb % 16 || cb < 256 || cb > c->stage_bytes) return none;
-  const uint64_t warps = threads / 32, per_warp = c->stage_bytes / warps;
-  uint64_t P;
-  if (sh.halo) {
-    // window of at most P c + 2 halo + 6 elements (16-byte widened), then P
-    // chunks of output.  The halo is re-read from L2 by every pass, so it
-    // must stay small against the pass: at most a quarter of it (a 2-D grid
-    // of 4096-wide rows needs two 16 KB halo rows per pass, and measured
-    // slower staged: 0.21 against 0.25 for dynamic(256)).  A stencil unit
-    // costs an owner lane several times an axpy unit, so long chunks walked
-    // by one lane lose (1-D, n = 2^26: c = 64 0.94 staged against 0.69,
-    // c = 128 0.74 against 0.65, c = 256 0.59 against 0.68): chunks of at
-    // most 512 bytes.
-    if (reduction || cb > 512) return none;
-    const uint64_t fixed = (2 * sh.halo + 8) * sh.elem;
-    P = per_warp > fixed ? (per_warp - fixed) / (2 * cb) : 0;
-    if (P > 32) P = 32;
-    if (P == 0 || 8 * sh.halo * sh.elem > P * cb) return none;
-  } else {
-    P = per_warp / (sh.arrays * cb);
-    if (P > 32) P = 32;
-    if (reduction ? (P < 32 || sh.arrays * cb > 512) : P < 16) return none;
-  }
-  // equal passes: a claim of 32 chunks in ceil(32 / P) passes of (nearly)
-  // the same size, not P, P, ..., remainder
-  P = (32 + (32 + P - 1) / P - 1) / ((32 + P - 1) / P);
-  const uint64_t wb = sh.halo ? ((P * chunk + 2 * sh.halo + 8) * sh.elem + 15) / 16 * 16 + P * cb
-                              : P * sh.arrays * cb;
-  // leave room for the kernel's static shared memory
-  if (smem_base + warps * wb + 2048 > (uint64_t)c->max_smem_optin) return none;
-  return {(uint32_t)P, (uint32_t)wb};
-}
-
-// The row form (region_rows.cuh) of a launch whose threads run contiguous
-// pieces.  It takes the launches below, measured on GB300 with axpy and dot at
-// n = 2^18 .. 2^26 (plain -> rows; G x T teams x threads):
-//   - pieces of 128 bytes on under static(c) and dynamic(c) (static(32)
-//     608 x 256: 260 -> 150 us, static(64) 191 -> 135; static(16) 232 -> 236),
-//     of 256 under static, whose short pieces still share lines (53 elements
-//     26.1 -> 28.4 us, 110 elements 45.9 -> 43.1);
-//   - blocks of 16 chunks on: with fewer, most lanes of the only claim are
-//     idle and each walks its chunk slab by slab (7 chunks of 256:
-//     11.2 -> 12.6 us; 27 chunks: 19.4 -> 13.4);
-//   - not static with a compensated sum: there the adds, not the loads, hold a
-//     launch (dot 500 x 512: 101 -> 111 us), unless the pieces are long;
-//   - a single stage a warp (teams of 1024) only where the plain form is
-//     worst: pieces of 512 bytes on (dynamic(256) 333 x 1024: 261 -> 164 us;
-//     static(64) 156 -> 175).
-// Shape: rows of 128 bytes where two stages a warp fit, else of 64; 64 also
-// for compensated sums, which want more warps (dot dynamic(256): 112 -> 103
-// us).  CTAs an SM: the count whose last wave is fullest, among those that
-// keep enough in flight (14 stages of 128-byte rows an SM; 608 x 256: one CTA
-// with two stages a warp 139 us, two with one 153).  Sized from the device's
-// shared memory, whatever the staging bytes; those at zero turn it off.
-struct RowPlan {
-  uint32_t row_bytes, stages;  // row_bytes 0: not this form
-  size_t smem;                 // dynamic shared memory of the buffers
-};
-static RowPlan row_plan(const omprt_ctx* c, const omprt_loop_desc* d, const StageShape& sh,
-                        uint64_t n, int ksched, uint64_t chunk, uint32_t teams, uint32_t threads,
-                        size_t smem_base, bool comp_sum) {
-  RowPlan best = {0u, 0u, 0};
-  if (!sh.arrays || sh.halo || c->stage_bytes == 0 || n == 0) return best;
-  uintptr_t mis = (uintptr_t)d->x;
-  if (sh.arrays == 2) mis |= (uintptr_t)d->y;
-  if (mis & 15) return best;
-  const bool whole = ksched == kStatic;  // one piece a thread
-  const uint64_t block = (n - 1) / teams + 1;
-  const uint64_t piece = (whole ? block / threads : chunk) * sh.elem;
-  if (piece < (whole ? (comp_sum ? 2048u : 256u) : 128u)) return best;
-  uint32_t warps = threads / 32;  // that can be busy at once
-  if (!whole) {
-    const uint64_t chunks = (block - 1) / chunk + 1;
-    if (chunks < 16) return best;
-    if ((chunks + 31) / 32 < warps) warps = (uint32_t)((chunks + 31) / 32);
-  }
-  constexpr uint64_t kStatic_ = 2048;      // the kernels' static shared memory, rounded up
-  constexpr uint64_t kReserved = 1024;     // what the hardware keeps of it for each CTA
-  const uint32_t most = threads >= 1024 ? 1 : 1024 / threads;  // CTAs an SM, by registers
-  double top = 0;
-  for (uint32_t row = comp_sum ? 64 : 128; row >= 64 && !best.row_bytes; row /= 2) {
-    const uint64_t set = (uint64_t)warps * rt::row_stage_bytes(sh.arrays, row);
-    for (uint32_t k = most; k >= 1; --k) {
-      uint64_t room = (uint64_t)c->smem_per_sm / k;
-      if (room > (uint64_t)c->max_smem_optin + kReserved) room = (uint64_t)c->max_smem_optin + kReserved;
-      const uint64_t fixed = kReserved + kStatic_ + smem_base;
-      uint64_t ns = room > fixed ? (room - fixed) / set : 0;
-      if (ns > rt::kRowStagesMax) ns = rt::kRowStagesMax;
-      if (ns == 0 || (ns == 1 && row == 128)) continue;
-      if (ns == 1 && threads >= 1024 && piece < 512) continue;
-      const double wave = (double)c->sm_count * k;
-      const double full = teams / wave / std::ceil(teams / wave);
-      const double flight = (double)(k * warps * ns) * row / (14 * 128), busy = k * warps / 16.0;
-      double score = full * std::fmin(flight, 1.0) * (ns > 1 ? 1.0 : 0.92);
-      if (comp_sum) score *= std::fmin(busy, 1.0);
-      if (score > top * 1.001) {
-        top = score;
-        best = {row, (uint32_t)ns, (size_t)(ns * set)};
-      }
-    }
-  }
-  return best;
 }
 
 static omprt_status launch_region_impl(omprt_ctx* c, const omprt_loop_desc* d, int64_t dist_chunk,
@@ -530,40 +402,20 @@ static omprt_status launch_region_impl(omprt_ctx* c, const omprt_loop_desc* d, i
     a.dyn_next = sl.dyn_next;
   }
   size_t smem = acc != kAccNone ? c->stack_bytes : 0;
-  // staged forms of dynamic(c), static(c) and static: the chunk a warp's
-  // lanes own (static without chunk: one block of n / (G T) per thread, used
-  // only when that division is exact, so every team's block is T of them)
-  uint64_t stage_c = 0;
-  if (ksched == kDynamic || ksched == kChunked || ksched == kNonmono) stage_c = (uint64_t)chunk;
-  if (ksched == kStatic && n % ((uint64_t)teams * (uint64_t)threads) == 0)
-    stage_c = n / ((uint64_t)teams * (uint64_t)threads);
   const StageShape sh = stage_shape(d, n);
-  // the staged form runs in blocks that start on a 16-byte boundary; where
-  // not all do, streaming bodies take the row form instead (axpy static(64)
-  // at n = 2^26, 900 x 128: 227 -> 139 us)
-  const bool aligned = n % (uint64_t)teams == 0 && n / (uint64_t)teams * sh.elem % 16 == 0;
-  if (stage_c && (aligned || d->body == OMPRT_BODY_STENCIL2D5)) {
-    const StagePlan sp = stage_plan(c, sh, stage_c, (uint32_t)threads, smem,
-                                    acc != kAccNone);
-    if (sp.chunks) {
-      a.stage_chunks = sp.chunks;
-      a.stage_warp_bytes = sp.warp_bytes;
-      a.stage_off = (uint32_t)smem;
-      if (ksched == kStatic) a.chunk = stage_c;
-      smem += (size_t)(threads / 32) * sp.warp_bytes;
-    }
-  }
-  if (!a.stage_chunks && (ksched == kStatic || ksched == kChunked || ksched == kDynamic ||
-                          ksched == kGuided || ksched == kNonmono)) {
-    const RowPlan rp = row_plan(c, d, sh, n, ksched, (uint64_t)chunk,
-                                (uint32_t)teams, (uint32_t)threads, smem, acc == kAccCompF32);
-    if (rp.row_bytes) {
-      a.row_bytes = rp.row_bytes;
-      a.row_stages = rp.stages;
-      a.stage_off = (uint32_t)smem;
-      smem += rp.smem;
-    }
-  }
+  const uintptr_t pointers = (uintptr_t)d->x | (sh.arrays == 2 ? (uintptr_t)d->y : 0);
+  const StreamPlan sp =
+      stream_plan({c->sm_count, c->max_smem_optin, c->smem_per_sm, c->stage_bytes}, sh,
+                  d->body == OMPRT_BODY_STENCIL2D5, (pointers & 15) == 0, n, ksched,
+                  (uint64_t)chunk, (uint32_t)teams, (uint32_t)threads, smem, acc != kAccNone,
+                  acc == kAccCompF32);
+  a.stage_chunks = sp.stage_chunks;
+  a.stage_warp_bytes = sp.stage_warp_bytes;
+  a.row_bytes = sp.row_bytes;
+  a.row_stages = sp.row_stages;
+  if (sp.stage_chunks) a.chunk = sp.stage_chunk;
+  if (sp.smem) a.stage_off = (uint32_t)smem;
+  smem += sp.smem;
   cudaStream_t st = (cudaStream_t)stream;
   cudaError_t e;
   if (d->body == OMPRT_BODY_STENCIL2D5 && ksched == kAuto && acc == kAccNone &&

@@ -12,11 +12,7 @@
 
 #include <cstdint>
 
-#ifdef __CUDACC__
-#define RT_HD __host__ __device__ __forceinline__
-#else
-#define RT_HD inline
-#endif
+#include "host_device.h"
 
 namespace rt {
 

@@ -3,9 +3,216 @@
 // Every rule states both sides as measured on GB300 (G x T: teams x threads).
 #pragma once
 
+#include <cmath>
+#include <cstddef>
 #include <cstdint>
 
+#include "host_device.h"
+
 namespace rt {
+
+// Schedules as the kernels are instantiated for them.
+enum : int { kStatic = 0, kChunked = 1, kDynamic = 2, kAuto = 3, kDist = 4, kGuided = 5,
+             kNonmono = 6 };
+
+// What a rule needs to know of the device and the context.
+struct PlanDevice {
+  int sm_count, max_smem_optin, smem_per_sm;
+  uint32_t stage_bytes;  // omprt_set_stage_bytes
+};
+
+// Arrays a body moves per iteration and their element size, for the staged
+// form of schedules (0 arrays: the body is not staged); halo: elements its
+// input window reaches beyond a pass on each side (the stencils).
+struct StageShape {
+  uint32_t arrays, elem;
+  uint64_t halo;
+};
+// Staged pass size for a dynamic(c) / static(c) / static launch: the largest
+// P <= 32 chunks whose buffers (every warp: P chunks of every array) fit the
+// context's per-team staging bytes, or 0 for the plain form.  Measured on
+// GB300 (n = 2^26): chunks below 256 bytes are already coalesced in the plain
+// form and lose to the per-pass overhead (static(8) axpy 0.94 staged against
+// 1.02 plain); without a reduction staging wins from P >= 16 (dynamic(256)
+// 0.97 against 0.64, static(64) 1.02 against 0.97) and loses below
+// (dynamic(1024): P <= 8); with a (compensated) reduction the per-element
+// work needs many warps per SM, and staging wins only with all 32 lanes busy
+// on chunks of at most 512 bytes over all arrays (dot dynamic(64) +16%, sum
+// +9%; dynamic(256) loses).
+struct StagePlan {
+  uint32_t chunks;      // P; 0: the plain form
+  uint32_t warp_bytes;  // shared memory per warp
+};
+inline StagePlan stage_plan(const PlanDevice& c, const StageShape& sh, uint64_t chunk,
+                            uint32_t threads, size_t smem_base, bool reduction) {
+  const StagePlan none = {0u, 0u};
+  if (!sh.arrays || c.stage_bytes == 0) return none;
+  const uint64_t cb = chunk * sh.elem;
+  if (cb % 16 || cb < 256 || cb > c.stage_bytes) return none;
+  const uint64_t warps = threads / 32, per_warp = c.stage_bytes / warps;
+  uint64_t P;
+  if (sh.halo) {
+    // window of at most P c + 2 halo + 6 elements (16-byte widened), then P
+    // chunks of output.  The halo is re-read from L2 by every pass, so it
+    // must stay small against the pass: at most a quarter of it (a 2-D grid
+    // of 4096-wide rows needs two 16 KB halo rows per pass, and measured
+    // slower staged: 0.21 against 0.25 for dynamic(256)).  A stencil unit
+    // costs an owner lane several times an axpy unit, so long chunks walked
+    // by one lane lose (1-D, n = 2^26: c = 64 0.94 staged against 0.69,
+    // c = 128 0.74 against 0.65, c = 256 0.59 against 0.68): chunks of at
+    // most 512 bytes.
+    if (reduction || cb > 512) return none;
+    const uint64_t fixed = (2 * sh.halo + 8) * sh.elem;
+    P = per_warp > fixed ? (per_warp - fixed) / (2 * cb) : 0;
+    if (P > 32) P = 32;
+    if (P == 0 || 8 * sh.halo * sh.elem > P * cb) return none;
+  } else {
+    P = per_warp / (sh.arrays * cb);
+    if (P > 32) P = 32;
+    if (reduction ? (P < 32 || sh.arrays * cb > 512) : P < 16) return none;
+  }
+  // equal passes: a claim of 32 chunks in ceil(32 / P) passes of (nearly)
+  // the same size, not P, P, ..., remainder
+  P = (32 + (32 + P - 1) / P - 1) / ((32 + P - 1) / P);
+  const uint64_t wb = sh.halo ? ((P * chunk + 2 * sh.halo + 8) * sh.elem + 15) / 16 * 16 + P * cb
+                              : P * sh.arrays * cb;
+  // leave room for the kernel's static shared memory
+  if (smem_base + warps * wb + 2048 > (uint64_t)c.max_smem_optin) return none;
+  return {(uint32_t)P, (uint32_t)wb};
+}
+
+constexpr uint32_t kRowStagesMax = 4;
+// bytes of one stage of one warp: 32 rows of every array, each padded by one
+// 16-byte unit (the lanes of a 128-bit access phase, one row apart, then hit
+// distinct banks), and one 16-byte record a lane
+constexpr RT_HD uint32_t row_stage_bytes(uint32_t arrays, uint32_t row) {
+  return 32u * (arrays * (row + 16u) + 16u);
+}
+
+// The row form (region_rows.cuh) of a launch whose threads run contiguous
+// pieces.  It takes the launches below, measured on GB300 with axpy and dot at
+// n = 2^18 .. 2^26 (plain -> rows; G x T teams x threads):
+//   - pieces of 128 bytes on under static(c) and dynamic(c) (static(32)
+//     608 x 256: 260 -> 150 us, static(64) 191 -> 135; static(16) 232 -> 236),
+//     of 256 under static, whose short pieces still share lines (53 elements
+//     26.1 -> 28.4 us, 110 elements 45.9 -> 43.1);
+//   - blocks of 16 chunks on: with fewer, most lanes of the only claim are
+//     idle and each walks its chunk slab by slab (7 chunks of 256:
+//     11.2 -> 12.6 us; 27 chunks: 19.4 -> 13.4);
+//   - not static with a compensated sum: there the adds, not the loads, hold a
+//     launch (dot 500 x 512: 101 -> 111 us), unless the pieces are long;
+//   - a single stage a warp (teams of 1024) only where the plain form is
+//     worst: pieces of 512 bytes on (dynamic(256) 333 x 1024: 261 -> 164 us;
+//     static(64) 156 -> 175).
+// Shape: rows of 128 bytes where two stages a warp fit, else of 64; 64 also
+// for compensated sums, which want more warps (dot dynamic(256): 112 -> 103
+// us).  CTAs an SM: the count whose last wave is fullest, among those that
+// keep enough in flight (14 stages of 128-byte rows an SM; 608 x 256: one CTA
+// with two stages a warp 139 us, two with one 153).  Sized from the device's
+// shared memory, whatever the staging bytes; those at zero turn it off.
+struct RowPlan {
+  uint32_t row_bytes, stages;  // row_bytes 0: not this form
+  size_t smem;                 // dynamic shared memory of the buffers
+};
+inline RowPlan row_plan(const PlanDevice& c, const StageShape& sh, bool aligned16, uint64_t n,
+                        int sched, uint64_t chunk, uint32_t teams, uint32_t threads,
+                        size_t smem_base, bool comp_sum) {
+  RowPlan best = {0u, 0u, 0};
+  if (!sh.arrays || sh.halo || c.stage_bytes == 0 || n == 0) return best;
+  if (!aligned16) return best;
+  const bool whole = sched == kStatic;  // one piece a thread
+  const uint64_t block = (n - 1) / teams + 1;
+  const uint64_t piece = (whole ? block / threads : chunk) * sh.elem;
+  if (piece < (whole ? (comp_sum ? 2048u : 256u) : 128u)) return best;
+  uint32_t warps = threads / 32;  // that can be busy at once
+  if (!whole) {
+    const uint64_t chunks = (block - 1) / chunk + 1;
+    if (chunks < 16) return best;
+    if ((chunks + 31) / 32 < warps) warps = (uint32_t)((chunks + 31) / 32);
+  }
+  constexpr uint64_t kStatic_ = 2048;      // the kernels' static shared memory, rounded up
+  constexpr uint64_t kReserved = 1024;     // what the hardware keeps of it for each CTA
+  const uint32_t most = threads >= 1024 ? 1 : 1024 / threads;  // CTAs an SM, by registers
+  double top = 0;
+  for (uint32_t row = comp_sum ? 64 : 128; row >= 64 && !best.row_bytes; row /= 2) {
+    const uint64_t set = (uint64_t)warps * row_stage_bytes(sh.arrays, row);
+    for (uint32_t k = most; k >= 1; --k) {
+      uint64_t room = (uint64_t)c.smem_per_sm / k;
+      if (room > (uint64_t)c.max_smem_optin + kReserved) room = (uint64_t)c.max_smem_optin + kReserved;
+      const uint64_t fixed = kReserved + kStatic_ + smem_base;
+      uint64_t ns = room > fixed ? (room - fixed) / set : 0;
+      if (ns > kRowStagesMax) ns = kRowStagesMax;
+      if (ns == 0 || (ns == 1 && row == 128)) continue;
+      if (ns == 1 && threads >= 1024 && piece < 512) continue;
+      const double wave = (double)c.sm_count * k;
+      const double full = teams / wave / std::ceil(teams / wave);
+      const double flight = (double)(k * warps * ns) * row / (14 * 128), busy = k * warps / 16.0;
+      double score = full * std::fmin(flight, 1.0) * (ns > 1 ? 1.0 : 0.92);
+      if (comp_sum) score *= std::fmin(busy, 1.0);
+      if (score > top * 1.001) {
+        top = score;
+        best = {row, (uint32_t)ns, (size_t)(ns * set)};
+      }
+    }
+  }
+  return best;
+}
+
+// Whether every team's block starts on a 16-byte boundary of the arrays: team
+// g's starts at g q + min(g, r), q = n / teams, r = n mod teams.
+inline bool blocks_aligned(uint64_t n, uint64_t teams, uint32_t elem) {
+  const uint64_t q = n / teams, r = n % teams;
+  if (r && (q + 1) * elem % 16) return false;                 // blocks 1 .. r
+  return r + 1 >= teams || q * elem % 16 == 0;                // those after
+}
+
+// Staged passes, rows, or (neither) the plain form.  aligned16: the arrays
+// start on a 16-byte boundary.
+struct StreamPlan {
+  uint32_t stage_chunks, stage_warp_bytes;  // staged form
+  uint64_t stage_chunk;                     // its chunk: the schedule's, or a thread's piece
+  uint32_t row_bytes, row_stages;           // row form
+  size_t smem;                              // dynamic shared memory beyond smem_base
+};
+inline StreamPlan stream_plan(const PlanDevice& c, const StageShape& sh, bool stencil2d,
+                              bool aligned16, uint64_t n, int sched, uint64_t chunk,
+                              uint32_t teams, uint32_t threads, size_t smem_base, bool reduction,
+                              bool comp_sum) {
+  StreamPlan p = {0u, 0u, 0u, 0u, 0u, 0};
+  // the chunk a warp's lanes own (static without chunk: one block of n / (G T)
+  // per thread, used only when that division is exact, so every team's block is
+  // T of them)
+  uint64_t stage_c = 0;
+  if (sched == kDynamic || sched == kChunked || sched == kNonmono) stage_c = chunk;
+  if (sched == kStatic && n % ((uint64_t)teams * threads) == 0)
+    stage_c = n / ((uint64_t)teams * threads);
+  // The staged form runs in blocks that start on a 16-byte boundary.  Where not
+  // all do, streaming bodies take the row form instead (axpy static(64) at n =
+  // 2^26, 900 x 128: 227 -> 139 us); where all do, whatever the remainder of the
+  // division, they stay (static(64), n = 2,050,019 on 3 x 64: 261 us staged, 402 in
+  // rows; dynamic(32) of int64 values, n = 256,999 on 4 x 64: 52 and 63).
+  if (stage_c && (stencil2d || blocks_aligned(n, teams, sh.elem))) {
+    const StagePlan sp = stage_plan(c, sh, stage_c, threads, smem_base, reduction);
+    if (sp.chunks) {
+      p.stage_chunks = sp.chunks;
+      p.stage_warp_bytes = sp.warp_bytes;
+      p.stage_chunk = stage_c;
+      p.smem = (size_t)(threads / 32) * sp.warp_bytes;
+      return p;
+    }
+  }
+  if (sched == kStatic || sched == kChunked || sched == kDynamic || sched == kGuided ||
+      sched == kNonmono) {
+    const RowPlan rp =
+        row_plan(c, sh, aligned16, n, sched, chunk, teams, threads, smem_base, comp_sum);
+    if (rp.row_bytes) {
+      p.row_bytes = rp.row_bytes;
+      p.row_stages = rp.stages;
+      p.smem = rp.smem;
+    }
+  }
+  return p;
+}
 
 // schedule(auto) 2-D stencil by strips of 64 columns a warp (k_stencil_cols.cu),
 // for grids the tensor tiles do not take; the others run in the region kernel.

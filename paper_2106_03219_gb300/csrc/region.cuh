@@ -7,12 +7,10 @@
 
 #include <type_traits>
 
+#include "plan.h"
 #include "rt_device.cuh"
 
 namespace rt {
-
-enum : int { kStatic = 0, kChunked = 1, kDynamic = 2, kAuto = 3, kDist = 4, kGuided = 5,
-             kNonmono = 6 };
 
 // Vectors each thread keeps in flight in the axpy body, and the largest team
 // the region kernels are compiled for (the register budget follows from it).

@@ -79,7 +79,6 @@ struct PieceGuided {  // a warp's guided claims
 // at once, which for a short block is fewer than its warps (a block of k
 // claims keeps k warps busy).  Under a static schedule those are the first
 // warps; under a dynamic one a warp takes a set with its first claim.
-constexpr uint32_t kRowStagesMax = 4;
 static __shared__ uint32_t rt_row_slots;
 
 // The elements [r0, r1) of one lane's row (array k at buf + k * arr, element 0
@@ -139,13 +138,6 @@ __device__ __forceinline__ void cp_async_wait(uint32_t newer) {
     case 2: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
     default: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
   }
-}
-
-// bytes of one stage of one warp: 32 rows of every array, each padded by one
-// 16-byte unit (the lanes of a 128-bit access phase, one row apart, then hit
-// distinct banks), and one 16-byte record a lane
-__host__ __device__ constexpr uint32_t row_stage_bytes(uint32_t arrays, uint32_t row) {
-  return 32u * (arrays * (row + 16u) + 16u);
 }
 
 template <uint32_t kRow, class Body, class Acc, class Pieces>

@@ -12,11 +12,33 @@ SOURCE = r"""
 #include "plan.h"
 using namespace rt;
 extern "C" {
+void stream(uint32_t arrays, uint32_t elem, uint64_t halo, int aligned16, uint64_t n, int sched,
+            uint64_t chunk, uint32_t teams, uint32_t threads, uint64_t smem_base, int reduction,
+            int comp_sum, uint32_t stage_bytes, uint64_t* out) {
+  const StreamPlan p = stream_plan({152, 232448, 233472, stage_bytes}, {arrays, elem, halo}, false,
+                                   aligned16, n, sched, chunk, teams, threads, smem_base,
+                                   reduction, comp_sum);
+  out[0] = p.stage_chunks;
+  out[1] = p.row_bytes;
+  out[2] = p.row_stages;
+  out[3] = p.smem;
+}
 int cols(uint64_t nx, uint64_t ny, uint32_t teams, uint32_t threads) {
   return cols_applies(nx, ny, teams, threads);
 }
 }
 """
+
+
+# schedules as plan.h numbers them
+STATIC, CHUNKED, DYNAMIC, AUTO, DIST, GUIDED, NONMONO = range(7)
+
+# body -> (arrays, element bytes, whether it reduces, whether by compensated adds)
+BODIES = {"axpy": (2, 4, False, False), "axpy_sum": (2, 4, True, True),
+          "axpy_i32_sum": (2, 4, True, False), "dot": (2, 4, True, True),
+          "load_f32_sum": (1, 4, True, True), "load_f32_max": (1, 4, True, False),
+          "load_bf16_sum": (1, 2, True, True), "load_i32": (1, 4, True, False),
+          "load_i64": (1, 8, True, False)}
 
 
 @functools.lru_cache(maxsize=None)
@@ -33,3 +55,20 @@ def _lib():
 def cols(nx, ny, teams, threads):
     """Whether a schedule(auto) 2-D stencil off the tensor tiles walks strips of columns."""
     return bool(_lib().cols(C.c_uint64(nx), C.c_uint64(ny), C.c_uint32(teams), C.c_uint32(threads)))
+
+
+def stream(body, n, sched, chunk, teams, threads, stage_bytes=32768, aligned16=True,
+           smem_base=None):
+    """The form of a streaming loop on a GB300: ("staged", chunks a pass), ("rows",
+    (bytes a row, stages)) or ("plain", None)."""
+    arrays, elem, red, comp = BODIES[body]
+    out = (C.c_uint64 * 4)()
+    base = (4096 if red else 0) if smem_base is None else smem_base
+    _lib().stream(arrays, elem, C.c_uint64(0), int(aligned16), C.c_uint64(n), sched,
+                  C.c_uint64(chunk), C.c_uint32(teams), C.c_uint32(threads), C.c_uint64(base),
+                  int(red), int(comp), C.c_uint32(stage_bytes), out)
+    if out[0]:
+        return "staged", out[0]
+    if out[1]:
+        return "rows", (out[1], out[2])
+    return "plain", None

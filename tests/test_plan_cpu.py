@@ -25,3 +25,32 @@ import plan_host as P
 ])
 def test_auto_stencil2d_strips(nx, ny, G, T, strips):
     assert P.cols(nx, ny, G, T) == strips
+
+
+@pytest.mark.parametrize("body,n,sched,chunk,G,T", [
+    ("axpy", 2_050_019, P.CHUNKED, 64, 3, 64),       # 261 us staged, 402 in rows, 394 plain
+    ("axpy", 135_387, P.DYNAMIC, 64, 1, 64),         # 65, 59, 99
+    ("axpy", 20_319, P.NONMONO, 256, 2, 32),         # 12, 16, 16
+    ("load_i64", 256_999, P.DYNAMIC, 32, 4, 64),     # 52, 63, 63
+    ("axpy", 300_007, P.DYNAMIC, 64, 1, 32),
+    ("load_i32", 300_007, P.CHUNKED, 64, 8, 64),     # 7 blocks of 37,501, one of 37,500
+    ("axpy", 1 << 26, P.DYNAMIC, 256, 4096, 32),
+])
+def test_staged_where_every_block_starts_on_16_bytes(body, n, sched, chunk, G, T):
+    q, r = divmod(n, G)
+    aligned = all((g * q + min(g, r)) * P.BODIES[body][1] % 16 == 0 for g in range(G))
+    assert (P.stream(body, n, sched, chunk, G, T)[0] == "staged") == aligned
+    assert P.stream(body, n, sched, chunk, G, T, stage_bytes=0)[0] == "plain"
+    assert P.stream(body, n + 16 * G, sched, chunk, G, T)[0] == \
+        P.stream(body, n, sched, chunk, G, T)[0]
+
+
+@pytest.mark.parametrize("body,elem", [("axpy", 4), ("load_i64", 8)])
+def test_blocks_aligned_is_exact(body, elem):
+    """The rule for blocks that start on 16 bytes against every block's start."""
+    for G in (1, 2, 3, 4, 5, 7, 8, 12):
+        for n in range(G * 2560, G * 2563):
+            q, r = divmod(n, G)
+            aligned = all((g * q + min(g, r)) * elem % 16 == 0 for g in range(G))
+            assert (P.stream(body, n, P.DYNAMIC, 256 // elem, G, 32)[0] == "staged") == aligned, \
+                (G, n)
