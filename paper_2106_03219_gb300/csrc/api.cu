@@ -288,21 +288,21 @@ omprt_status omprt_set_stencil_stage_bytes(omprt_ctx* c, int64_t bytes) {
 static StageShape stage_shape(const omprt_loop_desc* d, uint64_t n) {
   switch (d->body) {
     case OMPRT_BODY_AXPY:
-      return {2u, 4u, 0};  // f32 or i32: x, y (y written back)
+      return {2u, 4u, 0, true};  // f32 or i32: x, y (y written back)
     case OMPRT_BODY_DOT:
-      return {2u, 4u, 0};
+      return {2u, 4u, 0, false};
     case OMPRT_BODY_NONE:
-      if (d->data_type == OMPRT_F32 || d->data_type == OMPRT_I32) return {1u, 4u, 0};
-      if (d->data_type == OMPRT_BF16) return {1u, 2u, 0};
-      if (d->data_type == OMPRT_I64) return {1u, 8u, 0};
-      return {0u, 0u, 0};
+      if (d->data_type == OMPRT_F32 || d->data_type == OMPRT_I32) return {1u, 4u, 0, false};
+      if (d->data_type == OMPRT_BF16) return {1u, 2u, 0, false};
+      if (d->data_type == OMPRT_I64) return {1u, 8u, 0, false};
+      return {0u, 0u, 0, false};
     case OMPRT_BODY_STENCIL1D3:  // the window is read in 16-byte units
-      return n % 4 == 0 ? StageShape{1u, 4u, 1} : StageShape{0u, 0u, 0};
+      return n % 4 == 0 ? StageShape{1u, 4u, 1, true} : StageShape{0u, 0u, 0, false};
     case OMPRT_BODY_STENCIL2D5:  // and a unit must not straddle two rows
-      return n % 4 == 0 && d->nx % 4 == 0 ? StageShape{1u, 4u, (uint64_t)d->nx}
-                                          : StageShape{0u, 0u, 0};
+      return n % 4 == 0 && d->nx % 4 == 0 ? StageShape{1u, 4u, (uint64_t)d->nx, true}
+                                          : StageShape{0u, 0u, 0, false};
     default:
-      return {0u, 0u, 0};
+      return {0u, 0u, 0, false};
   }
 }
 

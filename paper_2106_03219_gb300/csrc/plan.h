@@ -27,6 +27,7 @@ struct PlanDevice {
 struct StageShape {
   uint32_t arrays, elem;
   uint64_t halo;
+  bool writes;  // the last array is written back
 };
 // Staged pass size for a dynamic(c) / static(c) / static launch: the largest
 // P <= 32 chunks whose buffers (every warp: P chunks of every array) fit the
@@ -89,13 +90,56 @@ constexpr RT_HD uint32_t row_stage_bytes(uint32_t arrays, uint32_t row) {
   return 32u * (arrays * (row + 16u) + 16u);
 }
 
-// The row form (region_rows.cuh) of a launch whose threads run contiguous
-// pieces.  It takes the launches below, measured on GB300 with axpy and dot at
-// n = 2^18 .. 2^26 (plain -> rows; G x T teams x threads):
-//   - pieces of 128 bytes on under static(c) and dynamic(c) (static(32)
-//     608 x 256: 260 -> 150 us, static(64) 191 -> 135; static(16) 232 -> 236),
-//     of 256 under static, whose short pieces still share lines (53 elements
-//     26.1 -> 28.4 us, 110 elements 45.9 -> 43.1);
+// Whether a launch that could take the row form (region_rows.cuh) gains by it.
+// Rows cost a trip through shared memory and each warp walks its slabs one after
+// another; the plain form has every lane read 32 bytes of its own piece.  The
+// plain form loses where that costs most: arrays from DRAM (many open pages),
+// pieces whose starts lie a multiple of 128 bytes apart (a warp's 32 lines then
+// compete for few sets of L1), two arrays and one written.  Measured plain -> rows
+// (us, G x T teams x threads), over 2839 random launches:
+//   - Maps, and integer sums with them: rows, but not under static with pieces
+//     below 400 bytes (axpy 608 x 256, 304 bytes 37.1 -> 43.3, 500 bytes 45.9 ->
+//     43.1), nor where pieces are no multiple of 128 bytes and short (static(50)
+//     608 x 256 n = 5.1 M 15.4 -> 23.9, static(100) n = 18 M 51.7 -> 54.9, dynamic(40)
+//     1 x 128 616 -> 799; static(200) n = 4.6 M 15.6 -> 12.0), or a warp's share is
+//     below 8 KB (nonmonotonic(50) 623 x 128 n = 2.8 M 17.1 -> 27.9).
+//   - Reads (sums, max, min, dot), whose plain form has no write-back: from L2 the
+//     plain form is faster (max static(4096) 23 x 32 n = 6.6 M 112 -> 176, int64
+//     static(50) 6 x 32 180 -> 396, bf16 static 9 x 32 136 -> 262), from DRAM rows
+//     are (max static 153 x 64 n = 58 M 138 -> 79, int32 static(1000) 15 x 256 n = 7.8 M
+//     100 -> 60).  26 MB of arrays are a fifth of the L2: they are still there from
+//     the launch before.  Under dynamic and nonmonotonic, pieces a multiple of 128
+//     bytes gain from L2 too with six warps a team (dot dynamic(128) 2 x 512, 492 -> 231).
+//   - Compensated sums inside a map: as reads, but always under dynamic schedules.
+//   - bf16: only dynamic and static chunks of a multiple of 128 bytes with six warps
+//     a team (static(64) 608 x 256 n = 19 M 26.4 -> 19.7; static(256) n = 3.2 M 9.7 ->
+//     13.1; nonmonotonic(100) n = 61 M 1259 -> 1562).
+// warps: a team's that can be busy; an_sm: of those on an SM at once; row: bytes.
+inline bool rows_gain(const StageShape& sh, int sched, uint64_t n, uint64_t chunk, uint64_t block,
+                      uint64_t piece, uint32_t warps, double an_sm, uint32_t row, bool comp_sum) {
+  const uint64_t bytes = n * sh.elem * sh.arrays, share = block * sh.elem / warps;
+  const bool whole = sched == kStatic, guided = sched == kGuided;
+  const bool claims = sched == kDynamic || sched == kNonmono;
+  const bool even = !whole && chunk * sh.elem % 128 == 0, dram = bytes > 26000000;
+  if (sh.writes && !comp_sum) {
+    if (whole) return piece >= 400;
+    if (guided || even) return true;
+    return claims ? share >= 8192 : piece >= 600 || (dram && an_sm <= 3);
+  }
+  if (sh.elem == 2) return !whole && !guided && even && warps >= 6;
+  if (whole) return dram && piece >= 640;
+  if (guided) return dram && (comp_sum || an_sm <= 6.3);
+  if (sh.writes) return claims || bytes > 40000000 || (even && an_sm > 0.4);
+  if (even) return claims ? dram || warps >= 6 : bytes > 40000000;
+  if (claims)
+    return comp_sum ? bytes > 77000000 : dram && (share >= 24u * 32 * row || piece >= 2000);
+  return bytes > 40000000 && piece >= 400 && an_sm <= 8;
+}
+
+// The row form of a launch whose threads run contiguous pieces: where it gains
+// (above), with
+//   - pieces of 128 bytes on under static(c) and dynamic(c) (axpy static(32)
+//     608 x 256: 260 -> 150 us; static(16) 232 -> 236);
 //   - blocks of 16 chunks on: with fewer, most lanes of the only claim are
 //     idle and each walks its chunk slab by slab (7 chunks of 256:
 //     11.2 -> 12.6 us; 27 chunks: 19.4 -> 13.4);
@@ -134,6 +178,7 @@ inline RowPlan row_plan(const PlanDevice& c, const StageShape& sh, bool aligned1
   constexpr uint64_t kReserved = 1024;     // what the hardware keeps of it for each CTA
   const uint32_t most = threads >= 1024 ? 1 : 1024 / threads;  // CTAs an SM, by registers
   double top = 0;
+  uint32_t ctas = 1;  // an SM
   for (uint32_t row = comp_sum ? 64 : 128; row >= 64 && !best.row_bytes; row /= 2) {
     const uint64_t set = (uint64_t)warps * row_stage_bytes(sh.arrays, row);
     for (uint32_t k = most; k >= 1; --k) {
@@ -151,10 +196,15 @@ inline RowPlan row_plan(const PlanDevice& c, const StageShape& sh, bool aligned1
       if (comp_sum) score *= std::fmin(busy, 1.0);
       if (score > top * 1.001) {
         top = score;
+        ctas = k;
         best = {row, (uint32_t)ns, (size_t)(ns * set)};
       }
     }
   }
+  const double an_sm = (double)warps * std::fmin(teams, (double)c.sm_count * ctas) / c.sm_count;
+  if (best.row_bytes && !rows_gain(sh, sched, n, chunk, block, piece, warps, an_sm,
+                                   best.row_bytes, comp_sum))
+    return {0u, 0u, 0};
   return best;
 }
 

@@ -12,10 +12,10 @@ SOURCE = r"""
 #include "plan.h"
 using namespace rt;
 extern "C" {
-void stream(uint32_t arrays, uint32_t elem, uint64_t halo, int aligned16, uint64_t n, int sched,
+void stream(uint32_t arrays, uint32_t elem, int writes, int aligned16, uint64_t n, int sched,
             uint64_t chunk, uint32_t teams, uint32_t threads, uint64_t smem_base, int reduction,
             int comp_sum, uint32_t stage_bytes, uint64_t* out) {
-  const StreamPlan p = stream_plan({152, 232448, 233472, stage_bytes}, {arrays, elem, halo}, false,
+  const StreamPlan p = stream_plan({152, 232448, 233472, stage_bytes}, {arrays, elem, 0, writes != 0}, false,
                                    aligned16, n, sched, chunk, teams, threads, smem_base,
                                    reduction, comp_sum);
   out[0] = p.stage_chunks;
@@ -64,7 +64,7 @@ def stream(body, n, sched, chunk, teams, threads, stage_bytes=32768, aligned16=T
     arrays, elem, red, comp = BODIES[body]
     out = (C.c_uint64 * 4)()
     base = (4096 if red else 0) if smem_base is None else smem_base
-    _lib().stream(arrays, elem, C.c_uint64(0), int(aligned16), C.c_uint64(n), sched,
+    _lib().stream(arrays, elem, int(body.startswith("axpy")), int(aligned16), C.c_uint64(n), sched,
                   C.c_uint64(chunk), C.c_uint32(teams), C.c_uint32(threads), C.c_uint64(base),
                   int(red), int(comp), C.c_uint32(stage_bytes), out)
     if out[0]:

@@ -54,3 +54,28 @@ def test_blocks_aligned_is_exact(body, elem):
             aligned = all((g * q + min(g, r)) * elem % 16 == 0 for g in range(G))
             assert (P.stream(body, n, P.DYNAMIC, 256 // elem, G, 32)[0] == "staged") == aligned, \
                 (G, n)
+
+
+@pytest.mark.parametrize("body,n,sched,chunk,G,T,rows", [  # plain and rows in us
+    ("load_i64", 1_411_583, P.CHUNKED, 50, 6, 32, False),       # 180, 396
+    ("load_bf16_sum", 5_276_959, P.STATIC, 0, 9, 32, False),    # 136, 262
+    ("load_f32_max", 6_639_461, P.CHUNKED, 4096, 23, 32, False),  # 112, 176
+    ("load_i32", 12_784_957, P.DYNAMIC, 40, 608, 256, False),   # 20.3, 30.5
+    ("load_i64", 428_377, P.DYNAMIC, 50, 1, 32, False),         # 452, 710
+    ("load_bf16_sum", 9_407_331, P.DYNAMIC, 100, 35, 1024, False),  # 26.6, 38.2
+    ("dot", 785_073, P.CHUNKED, 40, 2, 64, False),              # 242, 402
+    ("axpy_sum", 147_889, P.GUIDED, 256, 2, 32, False),         # 92, 136
+    ("axpy", 5_143_369, P.CHUNKED, 50, 608, 256, False),        # 15.4, 23.9
+    ("axpy", 3_030_322, P.CHUNKED, 40, 9, 32, False),           # 630, 789
+    ("axpy_i32_sum", 11_984_041, P.STATIC, 0, 608, 256, False),  # 37.1, 43.3
+    ("axpy", 67_108_864, P.DYNAMIC, 256, 608, 256, True),       # 197, 135
+    ("axpy", 50_000_001, P.STATIC, 0, 1184, 256, True),         # 124, 102
+    ("axpy_i32_sum", 1 << 20, P.STATIC, 0, 4, 128, True),       # 59.8, 53.7
+    ("axpy", 1_447_680, P.GUIDED, 64, 39, 256, True),           # 69.3, 14.6
+    ("dot", 30_055_685, P.DYNAMIC, 128, 18, 512, True),         # 491, 232
+    ("load_f32_max", 62_239_855, P.DYNAMIC, 128, 3, 1024, True),  # 3044, 1398
+    ("load_i32", 18_047_637, P.DYNAMIC, 4096, 26, 512, True),   # 140, 73
+    ("load_f32_max", 58_005_398, P.STATIC, 0, 153, 64, True),   # 138, 79
+])
+def test_rows_where_they_gain(body, n, sched, chunk, G, T, rows):
+    assert (P.stream(body, n, sched, chunk, G, T)[0] == "rows") == rows
