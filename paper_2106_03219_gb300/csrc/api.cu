@@ -534,8 +534,8 @@ static omprt_status launch_region_impl(omprt_ctx* c, const omprt_loop_desc* d, i
   // the 1-D stencil outside the staged form: each lane's next points staged
   if (d->body == OMPRT_BODY_STENCIL1D3 && acc == kAccNone && !a.stage_chunks &&
       c->stage_bytes != 0) {
-    e = launch_stencil1d_pieces(ksched, (unsigned)teams, (unsigned)threads, c->max_smem_optin, st,
-                                a);
+    e = launch_stencil1d_pieces(ksched, (unsigned)teams, (unsigned)threads, c->sm_count,
+                                c->max_smem_optin, c->smem_per_sm, st, a);
     if (e != cudaErrorNotSupported) return from_cuda(e);
     cudaGetLastError();
   }

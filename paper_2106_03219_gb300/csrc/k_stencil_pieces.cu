@@ -216,8 +216,6 @@ __device__ __forceinline__ void run_stencil_pieces(const BodyStencil2D& b,
 
 // 1-D 3-point stencil: the same slabs without rows above and below.  A lane's
 // row: the unit left of it, its NU units, the unit right of it, one of padding.
-constexpr uint32_t kLineNu = 8;
-constexpr uint32_t kLineStage = 32 * 16 * (kLineNu + 4);
 template <class Pieces>
 __device__ __forceinline__ void run_line_pieces(const BodyStencil1D& b, uint64_t bs,
                                                 Pieces& pieces) {
@@ -433,29 +431,16 @@ cudaError_t launch_stencil2d_pieces(int sched, unsigned teams, unsigned threads,
   }
 }
 
-// The 1-D stencil: chunks of 32 points on in blocks of 32 chunks (n = 2^26, 608 x
-// 256: static(64) 210 -> 129 us, dynamic(256) 151 -> 143, 500 x 512 187 -> 144; n =
-// 2^24 static(32) 78 -> 42, dynamic(64) 58 -> 36; n = 2^22 dynamic(256), 27 chunks a
-// block: 15.6 -> 16.1), and under static pieces of 64 to 256 points and from 1024
-// on (608 x 256: 107 points 42 -> 38 us, 431 points 123 -> 138; 148 x 128, 3542
-// points 222 -> 181).  Returns cudaErrorNotSupported, launching nothing, elsewhere.
-cudaError_t launch_stencil1d_pieces(int sched, unsigned teams, unsigned threads, int max_smem,
-                                    cudaStream_t st, const RegionArgs& a) {
-  const bool whole = sched == kStatic;
-  if ((sched != kStatic && sched != kChunked && sched != kDynamic && sched != kNonmono) ||
-      a.n == 0 || (((uintptr_t)a.x | (uintptr_t)a.out) & 15))
-    return cudaErrorNotSupported;
-  const uint64_t block = (a.n - 1) / teams + 1, piece = whole ? block / threads : a.chunk;
-  if (piece < (whole ? 64u : 32u) || (whole && piece > 256 && piece < 1024))
-    return cudaErrorNotSupported;
-  uint32_t warps = threads / 32;  // that can be busy at once
-  if (!whole) {
-    const uint64_t chunks = (block - 1) / a.chunk + 1;
-    if (chunks < 32) return cudaErrorNotSupported;
-    if ((chunks + 31) / 32 < warps) warps = (uint32_t)((chunks + 31) / 32);
-  }
-  const size_t smem = (size_t)warps * kLineStage;
-  if ((int64_t)smem > (int64_t)max_smem - 1024) return cudaErrorNotSupported;
+// The 1-D stencil.  Returns cudaErrorNotSupported, launching nothing, where the rule
+// (plan.h) leaves the launch to the other forms.
+cudaError_t launch_stencil1d_pieces(int sched, unsigned teams, unsigned threads, int sm_count,
+                                    int max_smem, int smem_per_sm, cudaStream_t st,
+                                    const RegionArgs& a) {
+  const LinePlan p = line_plan({sm_count, max_smem, smem_per_sm, 0u},
+                               (((uintptr_t)a.x | (uintptr_t)a.out) & 15) == 0, a.n, sched, a.chunk,
+                               teams, threads);
+  if (!p.smem) return cudaErrorNotSupported;
+  const size_t smem = p.smem;
   const StencilPieceArgs P = {a, 0u, 0u};
   switch (sched) {
     case kStatic: return launch_pieces<kStatic, 0>(teams, threads, smem, st, P);

@@ -185,8 +185,9 @@ cudaError_t launch_stencil2d_pieces(int sched, unsigned teams, unsigned threads,
                                     bool row_ring, cudaStream_t st, const RegionArgs& a);
 
 // The 1-D stencil the same way (without rows above and below).
-cudaError_t launch_stencil1d_pieces(int sched, unsigned teams, unsigned threads, int max_smem,
-                                    cudaStream_t st, const RegionArgs& a);
+cudaError_t launch_stencil1d_pieces(int sched, unsigned teams, unsigned threads, int sm_count,
+                                    int max_smem, int smem_per_sm, cudaStream_t st,
+                                    const RegionArgs& a);
 
 // the same schedules, a team's whole block and a grid row on each side in shared
 // memory, at most `budget` bytes (k_stencil_window.cu); cudaErrorNotSupported

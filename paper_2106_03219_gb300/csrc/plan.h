@@ -264,6 +264,62 @@ inline StreamPlan stream_plan(const PlanDevice& c, const StageShape& sh, bool st
   return p;
 }
 
+// 1-D stencil by lanes' pieces (k_stencil_pieces.cu); smem 0: not this form.
+// A warp's slabs follow one another here too, so it takes many warps, or data
+// from DRAM.  Measured plain -> pieces (us, G x T teams x threads), n of 1177
+// random launches:
+//   - chunks of 32 points on in blocks of 32 chunks (n = 2^26, 608 x 256: static(64)
+//     210 -> 129, dynamic(256) 151 -> 143; n = 2^22 dynamic(256), 27 chunks a block:
+//     15.6 -> 16.1), and under static pieces of 64 to 256 points and from 1024 on
+//     (608 x 256: 431 points 123 -> 138; 148 x 128, 3542 points 222 -> 181);
+//   - static: teams of 384 threads, or 26 MB of arrays (a fifth of the L2) and a
+//     warp an SM (26 x 32, 2,356,909 points 58 -> 120);
+//   - static(c): three busy warps a team or 0.6 an SM (static(1000) 3 x 32 220 ->
+//     427, 46 -> 89), for chunks that are no multiple of 32 points 80 points and
+//     five warps or 26 MB, or 29 an SM (static(40) 6 x 64 173 -> 440);
+//   - dynamic and nonmonotonic: seven busy warps a team, or four an SM in blocks of
+//     48 chunks (dynamic(500) 18 x 32 81 -> 167, nonmonotonic(256) 164 x 512, 33
+//     chunks a block 12.3 -> 18.8); chunks that are no multiple of 32 points from 26
+//     MB and eight warps an SM on, 16 below 80 points (dynamic(40) 1 x 64 144 -> 315,
+//     nonmonotonic(50) 662 x 256 n = 67 M 258 -> 162).
+constexpr uint32_t kLineNu = 8;  // 16-byte units a row
+constexpr uint32_t kLineStage = 32 * 16 * (kLineNu + 4);
+struct LinePlan {
+  size_t smem;
+};
+inline LinePlan line_plan(const PlanDevice& c, bool aligned16, uint64_t n, int sched,
+                          uint64_t chunk, uint32_t teams, uint32_t threads) {
+  const LinePlan none = {0};
+  const bool whole = sched == kStatic, claims = sched == kDynamic || sched == kNonmono;
+  if ((!whole && !claims && sched != kChunked) || n == 0 || !aligned16) return none;
+  const uint64_t block = (n - 1) / teams + 1, piece = whole ? block / threads : chunk;
+  if (piece < (whole ? 64u : 32u) || (whole && piece > 256 && piece < 1024)) return none;
+  uint32_t warps = threads / 32;  // that can be busy at once
+  uint64_t chunks = threads;
+  if (!whole) {
+    chunks = (block - 1) / chunk + 1;
+    if (chunks < 32) return none;
+    if ((chunks + 31) / 32 < warps) warps = (uint32_t)((chunks + 31) / 32);
+  }
+  const size_t smem = (size_t)warps * kLineStage;
+  if ((int64_t)smem > (int64_t)c.max_smem_optin - 1024) return none;
+  // CTAs and busy warps an SM at once
+  const double ctas = std::fmin(threads < 1024 ? 1024 / threads : 1,
+                                std::floor((double)c.smem_per_sm / (double)(smem + 1024)));
+  const double an_sm = warps * std::fmin(teams, c.sm_count * ctas) / c.sm_count;
+  const bool dram = n * 8 > 26000000, even = chunk % 32 == 0;
+  bool gain;
+  if (whole)
+    gain = threads >= 384 || (dram && an_sm >= 1);
+  else if (!claims)
+    gain = even ? warps >= 3 || an_sm > 0.6
+                : (piece >= 80 && (dram || warps >= 5)) || an_sm >= 29;
+  else
+    gain = even ? warps >= 7 || (an_sm >= 4 && chunks >= 48)
+                : dram && an_sm >= (piece >= 80 ? 8 : 16);
+  return gain ? LinePlan{smem} : none;
+}
+
 // schedule(auto) 2-D stencil by strips of 64 columns a warp (k_stencil_cols.cu),
 // for grids the tensor tiles do not take; the others run in the region kernel.
 //   - Strips at least 0.4 full: the lanes beyond a narrow grid's columns idle

@@ -23,6 +23,9 @@ void stream(uint32_t arrays, uint32_t elem, int writes, int aligned16, uint64_t 
   out[2] = p.row_stages;
   out[3] = p.smem;
 }
+int line(uint64_t n, int sched, uint64_t chunk, uint32_t teams, uint32_t threads) {
+  return line_plan({152, 232448, 233472, 32768}, true, n, sched, chunk, teams, threads).smem != 0;
+}
 int cols(uint64_t nx, uint64_t ny, uint32_t teams, uint32_t threads) {
   return cols_applies(nx, ny, teams, threads);
 }
@@ -72,3 +75,9 @@ def stream(body, n, sched, chunk, teams, threads, stage_bytes=32768, aligned16=T
     if out[1]:
         return "rows", (out[1], out[2])
     return "plain", None
+
+
+def line(n, sched, chunk, teams, threads):
+    """Whether a 1-D stencil outside the staged form goes by lanes' pieces."""
+    return bool(_lib().line(C.c_uint64(n), sched, C.c_uint64(chunk), C.c_uint32(teams),
+                            C.c_uint32(threads)))

@@ -79,3 +79,22 @@ def test_blocks_aligned_is_exact(body, elem):
 ])
 def test_rows_where_they_gain(body, n, sched, chunk, G, T, rows):
     assert (P.stream(body, n, sched, chunk, G, T)[0] == "rows") == rows
+
+
+@pytest.mark.parametrize("n,sched,chunk,G,T,pieces", [  # plain and pieces in us
+    (1_515_221, P.CHUNKED, 40, 6, 64, False),       # 173, 440
+    (2_356_909, P.STATIC, 0, 26, 32, False),        # 58, 120
+    (902_283, P.CHUNKED, 1000, 3, 32, False),       # 220, 427
+    (239_777, P.DYNAMIC, 40, 1, 64, False),         # 144, 315
+    (1_778_248, P.DYNAMIC, 500, 18, 32, False),     # 81, 167
+    (1_382_429, P.NONMONO, 256, 164, 512, False),   # 12.3, 18.8
+    (5_700_616, P.DYNAMIC, 256, 608, 256, False),   # 17.1, 21.3
+    (3_459_739, P.DYNAMIC, 50, 426, 1024, False),   # 16.6, 23.1
+    (1 << 26, P.CHUNKED, 64, 608, 256, True),       # 210, 129
+    (1 << 26, P.DYNAMIC, 256, 608, 256, True),      # 151, 143
+    (1 << 24, P.CHUNKED, 32, 608, 256, True),       # 78, 42
+    (1 << 24, P.DYNAMIC, 64, 608, 256, True),       # 58, 36
+    (66_684_445, P.NONMONO, 50, 662, 256, True),    # 258, 162
+])
+def test_stencil1d_pieces_where_they_gain(n, sched, chunk, G, T, pieces):
+    assert P.line(n, sched, chunk, G, T) == pieces
