@@ -30,8 +30,6 @@
 // is a team barrier reached by all threads from the same loop, so no thread
 // spins; the main thread's code between two regions is one step of its
 // program (a small state machine over (segment, phase)).
-#include <algorithm>
-
 #include "api_internal.h"
 
 namespace rt {
@@ -127,7 +125,6 @@ __device__ __forceinline__ float2 generic_for(const Body& body, uint64_t lo, uin
 // Tiles start on multiples of 4 elements; the array's last n % 4 elements,
 // which no whole 16-byte unit holds, run from global memory.
 // ---------------------------------------------------------------------------
-constexpr uint32_t kTilesMax = 8;
 static __shared__ __align__(8) uint64_t rt_tile_full[kTilesMax], rt_tile_empty[kTilesMax];
 static __shared__ int rt_tile_stop;
 constexpr int kAccs = 2;
@@ -412,8 +409,8 @@ __global__ void __launch_bounds__(1024) generic_kernel(const GenericArgs A) {
 
 // The tiled form's kernel: the team is threads 0 .. T - 1, the feeder a warp
 // beside it (T = blockDim.x - 32), and the team's barriers are named ones.  Its
-// loops need more than the 64 registers that teams of 1024 leave a thread.
-constexpr uint32_t kTiledThreads = 480;  // largest team: 128 registers a thread with the feeder
+// loops need more than the 64 registers that teams of 1024 leave a thread (98,
+// which is four warps in each quarter of an SM).
 __global__ void __launch_bounds__(kTiledThreads + 32) generic_tiled_kernel(const GenericArgs A) {
   enter_region_grid();
   __shared__ WorkDesc s_work;  // the team-shared hand-over word
@@ -520,24 +517,17 @@ extern "C" omprt_status omprt_launch_generic(omprt_ctx* c, const int64_t* seg_de
   a.pool = c->pool_dev;
   a.result = result_dev;
   a.status = c->status_dev;
-  // The tile ring takes what the teams resident on an SM leave each: at least
-  // three tiles, of 8192 elements (64 KB) if they fit, else of 4096, 2048 or
-  // 1024.  A tile costs a wait and an arrival a warp (4096 uneven segments, one
-  // team an SM: 206 us with 8192 elements, 250 with 4096).
-  const int per_sm =
-      std::max(1, std::min({(teams + c->sm_count - 1) / c->sm_count, 1024 / (threads + 32), 4}));
-  const int64_t room = std::min(c->smem_per_sm / per_sm - 1024, c->max_smem_optin) -
-                       (int64_t)a.stack_bytes - 1024;
-  a.ring_off = (a.stack_bytes + 127u) & ~127u;
-  a.tile_log2 = 13;
-  while (a.tile_log2 > 10 && room < 3 * (8 << a.tile_log2)) --a.tile_log2;
-  const int64_t fit = std::min<int64_t>(room > 0 ? room / (8 << a.tile_log2) : 0, kTilesMax);
-  a.tiles = (uint32_t)fit;
+  const uintptr_t xa = (uintptr_t)d->x, ya = (uintptr_t)d->y;
   // Tiles are loaded segments ahead: not where a segment's y is another's x
   // (arrays that overlap without being the same).
-  const uintptr_t xa = (uintptr_t)d->x, ya = (uintptr_t)d->y;
   const bool overlap_xy = xa != ya && (xa < ya ? ya - xa : xa - ya) < n * 4;
-  if (fit < 2 || threads > (int)kTiledThreads || ((xa | ya) & 15) || overlap_xy) {
+  const TilePlan p = tile_plan({c->sm_count, c->max_smem_optin, c->smem_per_sm, 0u}, a.stack_bytes,
+                               n, a.nseg, program == OMPRT_GENERIC_REDUCE && d->body == OMPRT_BODY_DOT,
+                               (uint32_t)teams, (uint32_t)threads);
+  a.ring_off = p.ring_off;
+  a.tile_log2 = p.tile_log2;
+  a.tiles = p.tiles;
+  if (!p.tiles || ((xa | ya) & 15) || overlap_xy) {
     static const size_t static_bytes = static_smem_of(generic_kernel);
     if (smem_optin(generic_kernel, a.stack_bytes, static_bytes) != cudaSuccess) {
       cudaGetLastError();

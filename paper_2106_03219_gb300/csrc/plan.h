@@ -320,6 +320,48 @@ inline LinePlan line_plan(const PlanDevice& c, bool aligned16, uint64_t n, int s
   return gain ? LinePlan{smem} : none;
 }
 
+// Generic regions by tiles (k_generic.cu); tiles 0: the plain form.
+// A tiled CTA is the team and its feeder warp, at 98 registers a thread: an SM holds
+// sixteen such warps, one team of 256 threads, three of 128, five of 64.  The ring
+// takes what the teams resident on an SM leave each, for at most four: at least
+// three tiles, of 8192 elements (64 KB) if they fit, else of 4096, 2048 or 1024.  A
+// tile costs a wait and an arrival a warp (4096 uneven segments, one team an SM:
+// 206 us with 8192 elements, 250 with 4096).
+//
+// Measured plain -> tiled (us, G x T teams x threads), 1000 random launches:
+//   - one wave of resident teams: tiled (152 x 256, 4096 segments of 13,000 elements
+//     434 -> 199; 18 x 32 2068 -> 292), but for single dots shorter than a thread
+//     each (152 x 256, 27 segments 4.0 -> 4.4);
+//   - more teams than are resident: a second wave starts cold, and teams of 256 run
+//     one after another where four plain ones share an SM (161 x 256 31 -> 52, 524 x 256
+//     42 -> 133, 2704 x 256 58 -> 184); up to 128 threads it pays from segments of 16
+//     elements a thread on (1765 x 32, segments of 13,000 418 -> 101, 960 x 128 of 3500
+//     47 -> 30, 3005 x 32 of 100 12 -> 30).
+constexpr uint32_t kTilesMax = 8;
+constexpr uint32_t kTiledThreads = 480;  // largest team, 512 threads with the feeder
+struct TilePlan {
+  uint32_t tiles, tile_log2, ring_off;  // ring_off: after the team stack
+};
+inline TilePlan tile_plan(const PlanDevice& c, uint32_t stack_bytes, uint64_t n, uint64_t nseg,
+                          bool single_dot, uint32_t teams, uint32_t threads) {
+  const TilePlan none = {0u, 0u, 0u};
+  if (threads > kTiledThreads || nseg == 0) return none;
+  const uint32_t sms = (uint32_t)c.sm_count, fit = 16 / (threads / 32 + 1) < 4
+                                                       ? 16 / (threads / 32 + 1) : 4;
+  const uint32_t want = (teams - 1) / sms + 1, resident = want < fit ? want : fit;
+  int64_t room = c.smem_per_sm / (int64_t)resident - 1024;
+  if (room > c.max_smem_optin) room = c.max_smem_optin;
+  room -= (int64_t)stack_bytes + 1024;
+  TilePlan p = {0u, 13u, (stack_bytes + 127u) & ~127u};
+  while (p.tile_log2 > 10 && room < 3 * (8 << p.tile_log2)) --p.tile_log2;
+  const int64_t tiles = room > 0 ? room / (8 << p.tile_log2) : 0;
+  if (tiles < 2) return none;
+  p.tiles = tiles < kTilesMax ? (uint32_t)tiles : kTilesMax;
+  const double a_thread = (double)n / (double)nseg / threads;  // a segment's elements
+  if (want <= fit) return single_dot && nseg <= teams && a_thread < 1 ? none : p;
+  return threads <= 128 && a_thread >= 16 ? p : none;
+}
+
 // schedule(auto) 2-D stencil by strips of 64 columns a warp (k_stencil_cols.cu),
 // for grids the tensor tiles do not take; the others run in the region kernel.
 //   - Strips at least 0.4 full: the lanes beyond a narrow grid's columns idle

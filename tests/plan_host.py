@@ -26,6 +26,10 @@ void stream(uint32_t arrays, uint32_t elem, int writes, int aligned16, uint64_t 
 int line(uint64_t n, int sched, uint64_t chunk, uint32_t teams, uint32_t threads) {
   return line_plan({152, 232448, 233472, 32768}, true, n, sched, chunk, teams, threads).smem != 0;
 }
+int tiles(uint64_t stack, uint64_t n, uint64_t nseg, int dot, uint32_t teams, uint32_t threads) {
+  return tile_plan({152, 232448, 233472, 32768}, (uint32_t)stack, n, nseg, dot, teams,
+                   threads).tiles;
+}
 int cols(uint64_t nx, uint64_t ny, uint32_t teams, uint32_t threads) {
   return cols_applies(nx, ny, teams, threads);
 }
@@ -81,3 +85,9 @@ def line(n, sched, chunk, teams, threads):
     """Whether a 1-D stencil outside the staged form goes by lanes' pieces."""
     return bool(_lib().line(C.c_uint64(n), sched, C.c_uint64(chunk), C.c_uint32(teams),
                             C.c_uint32(threads)))
+
+
+def tiles(n, nseg, teams, threads, single_dot=False, stack=4096):
+    """Tiles of a generic launch's ring; 0: the plain form."""
+    return _lib().tiles(C.c_uint64(stack), C.c_uint64(n), C.c_uint64(nseg), int(single_dot),
+                        C.c_uint32(teams), C.c_uint32(threads))

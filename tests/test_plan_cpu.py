@@ -98,3 +98,31 @@ def test_rows_where_they_gain(body, n, sched, chunk, G, T, rows):
 ])
 def test_stencil1d_pieces_where_they_gain(n, sched, chunk, G, T, pieces):
     assert P.line(n, sched, chunk, G, T) == pieces
+
+
+@pytest.mark.parametrize("nseg,avg,G,T,dot,tiled", [  # plain and tiled in us
+    (2226, 342, 161, 256, False, False),        # 31, 52
+    (9044, 36, 524, 256, True, False),          # 42, 133
+    (13_158, 150, 2704, 256, True, False),      # 58, 184
+    (182, 450, 2731, 256, False, False),        # 6.1, 24.2
+    (12_501, 5342, 546, 256, False, False),     # 277, 488
+    (6879, 94, 3005, 32, True, False),          # 11.6, 29.5
+    (9367, 66, 1251, 128, False, False),        # 34.8, 47.4
+    (27, 58, 152, 256, True, False),            # 4.0, 4.4
+    (4096, 13_280, 152, 256, False, True),      # 434, 199
+    (963, 10_000, 18, 32, True, True),          # 2068, 292
+    (568, 13_000, 1765, 32, False, True),       # 418, 101
+    (2370, 3505, 960, 128, False, True),        # 47, 30
+    (3906, 7800, 7, 128, False, True),          # 4199, 1407
+])
+def test_generic_tiles_where_they_gain(nseg, avg, G, T, dot, tiled):
+    assert (P.tiles(nseg * avg, nseg, G, T, dot) > 0) == tiled
+
+
+def test_generic_tile_rings_fit():
+    """Rings of every team size lie beside the stack in the shared memory of one SM."""
+    for T in range(32, 513, 32):
+        for G in (1, 152, 153, 304, 305, 456, 608, 5000):
+            for stack in (0, 4096, 48 * 1024, 150 * 1024, 226 * 1024):
+                t = P.tiles(1 << 30, 64, G, T, stack=stack)
+                assert t == 0 or 2 <= t <= 8 and T <= 480
