@@ -1,7 +1,6 @@
 // The C ABI (include/omprt.h): context, argument validation, schedule
 // resolution and kernel dispatch.  Host code only; every step of the loop
 // itself runs in the executor kernels.
-#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstring>
@@ -539,14 +538,9 @@ static omprt_status launch_region_impl(omprt_ctx* c, const omprt_loop_desc* d, i
     if (e != cudaErrorNotSupported) return from_cuda(e);
     cudaGetLastError();
   }
-  // A grid that leaves slots free on every SM would be overlapped unevenly: the
-  // next one's blocks fill those slots first, and SMs that finish early take the
-  // rest.  The point-by-point 2-D stencil is bound by instructions, so its
-  // fullest SM then sets the time; it goes plain there (1291 x 634 on 842 x 128:
-  // static(8) 8.6 us overlapped, 7.1 plain, static(1) 6.2 and 5.5).  Bound by
-  // memory, the other bodies gain 0.4 us by the overlap.
+  // the point-by-point 2-D stencil where an overlapped grid's blocks spread unevenly
   const bool uneven = d->body == OMPRT_BODY_STENCIL2D5 && ksched != kAuto &&
-                      teams > c->sm_count && teams < c->sm_count * std::max(1, 1024 / threads);
+                      overlap_uneven(n, ksched, (uint32_t)teams, (uint32_t)threads, c->sm_count);
   rt::OverlapScope even(c->launch_overlap && !uneven, (size_t)c->smem_per_sm);
   const bool f32path = d->data_type == OMPRT_F32 || d->data_type == OMPRT_BF16;
   if (d->body == OMPRT_BODY_MAP_RECORD || !f32path)

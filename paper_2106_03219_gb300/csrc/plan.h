@@ -362,6 +362,26 @@ inline TilePlan tile_plan(const PlanDevice& c, uint32_t stack_bytes, uint64_t n,
   return threads <= 128 && a_thread >= 16 ? p : none;
 }
 
+// Whether a grid of the region kernel's point-by-point 2-D stencil goes without
+// launch overlap.  An overlapped grid's first blocks fill the slots the one before
+// leaves free, and SMs that finish early take the rest, so its fullest SM can hold
+// more blocks than an even spread gives; bound by instructions, that SM sets the
+// time.  It matters where the SMs are nearly evenly filled and have slots for 1.1 to
+// 1.8 times the blocks, from four points a thread on, twelve under dist_schedule
+// (plain -> overlapped, us: static(8) 1291 x 634, 842 x 128 7.1 -> 8.6; static(1) with
+// 47 points a thread, five of eight slots, 18 -> 25; static 2205 wide, six of eight
+// 61 -> 77).  Everywhere else the overlap gains its microsecond or costs nothing
+// (static 1960 x 21, 161 x 256 2.3 -> 1.9; dist 461 x 145, 577 x 256 3.2 -> 2.8;
+// dynamic(8), two of eight slots, 4.7 -> 4.3).
+inline bool overlap_uneven(uint64_t n, int sched, uint32_t teams, uint32_t threads, int sm_count) {
+  if (teams <= (uint32_t)sm_count) return false;
+  const double an_sm = std::ceil((double)teams / sm_count);
+  const double slots = threads < 1024 ? 1024 / threads : 1;
+  const double full = teams / (sm_count * an_sm), spare = slots / an_sm;
+  return full >= 0.7 && spare >= 1.1 && spare < 1.8 &&
+         n >= (sched == kDist ? 12ull : 4ull) * teams * threads;
+}
+
 // schedule(auto) 2-D stencil by strips of 64 columns a warp (k_stencil_cols.cu),
 // for grids the tensor tiles do not take; the others run in the region kernel.
 //   - Strips at least 0.4 full: the lanes beyond a narrow grid's columns idle

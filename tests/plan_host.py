@@ -30,6 +30,9 @@ int tiles(uint64_t stack, uint64_t n, uint64_t nseg, int dot, uint32_t teams, ui
   return tile_plan({152, 232448, 233472, 32768}, (uint32_t)stack, n, nseg, dot, teams,
                    threads).tiles;
 }
+int uneven(uint64_t n, int sched, uint32_t teams, uint32_t threads) {
+  return overlap_uneven(n, sched, teams, threads, 152);
+}
 int cols(uint64_t nx, uint64_t ny, uint32_t teams, uint32_t threads) {
   return cols_applies(nx, ny, teams, threads);
 }
@@ -91,3 +94,8 @@ def tiles(n, nseg, teams, threads, single_dot=False, stack=4096):
     """Tiles of a generic launch's ring; 0: the plain form."""
     return _lib().tiles(C.c_uint64(stack), C.c_uint64(n), C.c_uint64(nseg), int(single_dot),
                         C.c_uint32(teams), C.c_uint32(threads))
+
+
+def uneven(n, sched, teams, threads):
+    """Whether the region kernel's 2-D stencil goes without launch overlap."""
+    return bool(_lib().uneven(C.c_uint64(n), sched, C.c_uint32(teams), C.c_uint32(threads)))

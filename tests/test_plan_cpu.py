@@ -126,3 +126,20 @@ def test_generic_tile_rings_fit():
             for stack in (0, 4096, 48 * 1024, 150 * 1024, 226 * 1024):
                 t = P.tiles(1 << 30, 64, G, T, stack=stack)
                 assert t == 0 or 2 <= t <= 8 and T <= 480
+
+
+@pytest.mark.parametrize("n,sched,G,T,plain", [  # without overlap and with, us
+    (1291 * 634, P.CHUNKED, 842, 128, True),        # 7.1, 8.6
+    (33 * 782 * 128, P.STATIC, 782, 128, True),     # 51, 64
+    (59 * 345 * 256, P.CHUNKED, 345, 256, True),    # 24, 29
+    (1960 * 21, P.STATIC, 161, 256, False),         # 2.3, 1.9
+    (3 * 4534, P.STATIC, 629, 32, False),           # 2.3, 1.8
+    (461 * 145, P.DIST, 577, 256, False),           # 3.2, 2.6
+    (1024 * 1024, P.CHUNKED, 2048, 32, False),      # 6.4, 5.8
+    (1024 * 1024, P.STATIC, 2048, 32, False),       # 6.2, 5.8
+    (22 * 12_345, P.DIST, 202, 64, False),          # 8.9, 8.3
+    (7 * 33_202, P.STATIC, 205, 128, False),        # 3.5, 3.3
+    (1 << 24, P.STATIC, 100, 256, False),           # less than a block an SM
+])
+def test_stencil2d_launch_overlap(n, sched, G, T, plain):
+    assert P.uneven(n, sched, G, T) == plain
