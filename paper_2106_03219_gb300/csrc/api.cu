@@ -486,7 +486,8 @@ static omprt_status launch_region_impl(omprt_ctx* c, const omprt_loop_desc* d, i
       c->stencil_stage_bytes != 0) {
     int budget = c->max_smem_optin - 2048;
     if ((int64_t)c->stencil_stage_bytes < budget) budget = (int)c->stencil_stage_bytes;
-    e = launch_stencil2d_window(ksched, (unsigned)teams, (unsigned)threads, budget, st, a);
+    e = launch_stencil2d_window(ksched, (unsigned)teams, (unsigned)threads, c->sm_count,
+                                c->smem_per_sm, budget, st, a);
     if (e != cudaErrorNotSupported) return from_cuda(e);
     cudaGetLastError();
     e = launch_stencil2d_pieces(ksched, (unsigned)teams, (unsigned)threads, c->max_smem_optin,

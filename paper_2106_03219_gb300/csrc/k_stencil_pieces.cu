@@ -388,15 +388,19 @@ static cudaError_t launch_pieces_nu(uint32_t nu, unsigned teams, unsigned thread
 // cudaErrorNotSupported, launching nothing, where this form does not apply or
 // loses to the others (4096^2 and 2048^2, plain or ring forms against this one,
 // G x T teams x threads):
-//   - pieces of 32 points on; teams of up to 512 threads;
+//   - pieces of 32 points on in blocks of 16 (dynamic(500), 174 x 122 on 6116 x 128,
+//     blocks of four points: 14 us point by point, 22 here); teams of up to 512
+//     threads;
 //   - odd grids (nx no multiple of 4): always (3001 x 2503, 608 x 256: static
 //     98 -> 37 us, static(32) 166 -> 45, static(128) 166 -> 31, static(500) 178
 //     -> 41, dynamic(64) 168 -> 34, dynamic(256) 180 -> 46);
 //   - other grids: static (608 x 256 68 -> 58, 900 x 128 85 -> 51), static(c) but
 //     for the c in [32, 128] of the row ring (static(64) 608 x 256: 65 there, 70
 //     here; static(500) 136 -> 55), nonmonotonic (608 x 256 94 -> 62), dynamic(c)
-//     with 48 chunks a block (dynamic(256) 608 x 256 95 -> 64, 900 x 128 107 ->
-//     59; but 2048^2, whose blocks hold one claim: 30 -> 37).
+//     with 102 chunks a block of whole 32 points (dynamic(256) 608 x 256 95 -> 64, 900 x
+//     128 107 -> 59; dynamic(500), 4096 x 28 on 4 x 64, 58 chunks: 18 -> 48;
+//     dynamic(100), 5492 x 1950 on 608 x 256 33 -> 48), or with 48 any in blocks beyond
+//     54,000 points, which no window holds (dynamic(1000) 86 x 64 458 -> 255).
 // Rows of 16 points under static and short chunks, whose many pieces want many
 // warps; of 32 under dynamic and from chunks of 256 on, and where 32 fit.  One
 // slab a warp: the same memory as two slabs of half the warps was slower
@@ -409,11 +413,14 @@ cudaError_t launch_stencil2d_pieces(int sched, unsigned teams, unsigned threads,
       (((uintptr_t)a.x | (uintptr_t)a.out) & 15))
     return cudaErrorNotSupported;
   const uint64_t block = (a.n - 1) / teams + 1;
-  if ((whole ? block / threads : a.chunk) < 32) return cudaErrorNotSupported;
+  if ((whole ? block / threads : a.chunk) < 32 || block < 16) return cudaErrorNotSupported;
   uint32_t warps = threads / 32;  // that can be busy at once
   if (!whole) {
     const uint64_t chunks = (block - 1) / a.chunk + 1;
-    if (!odd && chunks < (sched == kDynamic ? 48u : 16u)) return cudaErrorNotSupported;
+    if (!odd && chunks < (sched != kDynamic ? 16u : block > 54000 ? 48u : 102u))
+      return cudaErrorNotSupported;
+    if (!odd && sched == kDynamic && block <= 54000 && a.chunk % 32 != 0)
+      return cudaErrorNotSupported;
     if (!odd && sched == kChunked && a.chunk <= 128 && row_ring) return cudaErrorNotSupported;
     if ((chunks + 31) / 32 < warps) warps = (uint32_t)((chunks + 31) / 32);
   }

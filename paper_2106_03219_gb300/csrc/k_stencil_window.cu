@@ -215,33 +215,24 @@ static cudaError_t launch_window_odd(bool odd, unsigned teams, unsigned threads,
              : launch_window<SCHED, false>(teams, threads, smem, st, P);
 }
 
-// Returns cudaErrorNotSupported, launching nothing, where this form does not
-// apply (a window beyond `budget` bytes) or loses to the others: pieces under
-// 8 points (16 under static), and blocks under 1024 points on grids of whole
-// 16-byte units (700 x 600, static(64), 608 x 256: 6.0 us in the others, 6.7 here)
-// or with chunks under 32 (293 x 1034, static(8), 1142 x 256: 7.3, 8.8 here).
-cudaError_t launch_stencil2d_window(int sched, unsigned teams, unsigned threads, int budget,
-                                    cudaStream_t st, const RegionArgs& a) {
-  const bool whole = sched == kStatic, odd = a.nx % 4 != 0;
-  if ((sched != kStatic && sched != kChunked && sched != kDynamic && sched != kNonmono) ||
-      a.n == 0 || a.nx >= (1ull << 24) || a.ny >= (1ull << 31) || ((uintptr_t)a.x & 15) ||
-      ((uintptr_t)a.out & 31))
-    return cudaErrorNotSupported;
-  const uint64_t block = (a.n - 1) / teams + 1;
-  const uint64_t piece = whole ? block / threads : a.chunk;
-  if (piece < (whole ? 16u : 8u) || block > (1ull << 24) ||
-      (block < 1024 && (!odd || piece < 32)))
-    return cudaErrorNotSupported;
+// Returns cudaErrorNotSupported, launching nothing, where the rule (plan.h) leaves the
+// launch to the other forms.
+cudaError_t launch_stencil2d_window(int sched, unsigned teams, unsigned threads, int sm_count,
+                                    int smem_per_sm, int budget, cudaStream_t st,
+                                    const RegionArgs& a) {
+  const WindowPlan p =
+      window_plan({sm_count, 0, smem_per_sm, 0u}, budget,
+                  ((uintptr_t)a.x & 15) == 0 && ((uintptr_t)a.out & 31) == 0, a.nx, a.ny, sched,
+                  a.chunk, teams, threads);
+  if (!p.smem) return cudaErrorNotSupported;
+  const bool odd = a.nx % 4 != 0;
+  const size_t smem = p.smem;
   WindowArgs P;
   P.r = a;
   P.sn = (uint32_t)(4 - a.nx % 4) % 4;
   P.ss = (uint32_t)(a.nx % 4);
-  P.lead = (uint32_t)((a.nx + 7) / 8 * 8 + 8);
-  // block, rounded to sectors on both sides, a row and a sector on each side
-  const uint64_t floats = block + 16 + 2 * (uint64_t)P.lead + 8;
-  const size_t smem = (size_t)(floats + 3) / 4 * 16;
-  if ((int64_t)smem > budget) return cudaErrorNotSupported;
-  P.seg = (uint32_t)((floats + kSegs - 1) / kSegs + 3) / 4 * 4;
+  P.lead = p.lead;
+  P.seg = (uint32_t)((p.floats + kSegs - 1) / kSegs + 3) / 4 * 4;
   switch (sched) {
     case kStatic: return launch_window_odd<kStatic>(odd, teams, threads, smem, st, P);
     case kChunked: return launch_window_odd<kChunked>(odd, teams, threads, smem, st, P);

@@ -192,8 +192,9 @@ cudaError_t launch_stencil1d_pieces(int sched, unsigned teams, unsigned threads,
 // the same schedules, a team's whole block and a grid row on each side in shared
 // memory, at most `budget` bytes (k_stencil_window.cu); cudaErrorNotSupported
 // (nothing launched) where that form does not apply.
-cudaError_t launch_stencil2d_window(int sched, unsigned teams, unsigned threads, int budget,
-                                    cudaStream_t st, const RegionArgs& a);
+cudaError_t launch_stencil2d_window(int sched, unsigned teams, unsigned threads, int sm_count,
+                                    int smem_per_sm, int budget, cudaStream_t st,
+                                    const RegionArgs& a);
 
 // static(c) 2-D stencil with the team's rows staged through a ring in shared
 // memory (k_stencil_rows.cu): c in [4, 8) and [32, 128], where it beats the

@@ -382,6 +382,79 @@ inline bool overlap_uneven(uint64_t n, int sched, uint32_t teams, uint32_t threa
          n >= (sched == kDist ? 12ull : 4ull) * teams * threads;
 }
 
+// 2-D stencil by block windows (k_stencil_window.cu); smem 0: not this form, either
+// because it does not apply (a window beyond `budget` bytes, arrays off 16 and 32
+// bytes) or because it loses.  A team loads its block and two grid rows and runs
+// it with its own warps only, where the row ring and the streamed ring share rows
+// among the teams of a CTA and the plain form has every warp an SM holds.  Measured
+// others -> windows (us, G x T teams x threads), 1500 launches:
+//   - pieces under 8 points (16 under static) and blocks under 1024 points on grids
+//     of whole 16-byte units (700 x 600, static(64), 608 x 256: 6.0 -> 6.7) or with
+//     chunks under 32 (293 x 1034, static(8), 1142 x 256: 7.3 -> 8.8): others;
+//   - blocks under 16 points: others (dynamic(32), 5 x 1737 on 3378 x 256 13.7 -> 21.4);
+//   - pieces under 24 points on grids up to three columns wide (static(8), 3 x 444,749
+//     on 864 x 1024 17.0 -> 24.1), and where blocks and rows are whole 32-byte
+//     sectors, so that the plain form reads vectors: others (static(8), 4096^2 on
+//     8192 x 32 36 -> 88, on 1024 x 32 90 -> 176; static, 16 points a thread, 2048^2 on
+//     4096 x 64 12 -> 20); static(c) of such short pieces also on blocks under 1536
+//     points of large grids (static(16), 4096 x 47 on 188 x 1024 6.5 -> 9.0);
+//   - dynamic on grids of whole units, teams of up to 384 threads: the row ring and
+//     the streamed ring with twelve teams an SM on, but for small halos (4096^2,
+//     dynamic(100) on 8192 x 32 45 -> 74, on 2048 x 128 44 -> 45; dynamic(256) on 16,000
+//     x 32 105 -> 158), and where fewer than 77 lanes an SM get a chunk, but for short
+//     blocks of more than a row (dynamic(1000), 16 x 306,391 on 1091 x 64 52 -> 99,
+//     2048 x 39 on 39 x 32 14 -> 27; dynamic(256), 2236 x 398 on 525 x 256 20.7 ->
+//     14.8);
+//   - nonmonotonic with three and more rows a block and many waves: others (4096^2,
+//     nonmonotonic(100) on 16,000 x 32 80 -> 111).
+struct WindowPlan {
+  size_t smem;
+  uint64_t floats;  // the window's
+  uint32_t lead;    // of them before the block's first sector: nx rounded up to 8, and 8
+};
+inline bool window_gain(const PlanDevice& c, uint64_t nx, uint64_t n, int sched, uint64_t chunk,
+                        uint64_t piece, uint32_t teams, uint32_t threads, size_t smem) {
+  const uint64_t block = (n - 1) / teams + 1;
+  const bool whole = sched == kStatic, few = piece < 24, odd = nx % 4 != 0;
+  if (block < 16 || (few && nx <= 3)) return false;
+  if (few && (whole || sched == kChunked) && nx % 8 == 0 && n % (8ull * teams) == 0 &&
+      (!whole || n % (8ull * teams * threads) == 0))
+    return false;
+  if (few && sched == kChunked && block < 1536 && n > 800000) return false;
+  // rows of halo a block, resident CTAs an SM, lanes an SM that get a chunk
+  const double halo = 2.0 * (double)nx / (double)block;
+  const double fit = std::fmin(std::fmin(threads < 1024 ? 1024 / threads : 1, 32),
+                               std::fmax(1, std::floor((double)c.smem_per_sm / (smem + 1624.0))));
+  const double resident = std::fmin(fit, std::ceil((double)teams / c.sm_count));
+  if (sched == kNonmono) return halo <= 6 || teams <= 5 * c.sm_count * fit;
+  if (sched != kDynamic || odd || threads > 384) return true;
+  if (teams > 12u * (uint32_t)c.sm_count) return threads >= 64 && halo <= 1.5;
+  const uint64_t chunks = (block - 1) / chunk + 1;
+  const double lanes = resident * std::fmin((double)chunks, threads);
+  return lanes > 76 || (block <= 24ull * threads && halo > 0.12);
+}
+inline WindowPlan window_plan(const PlanDevice& c, int64_t budget, bool aligned, uint64_t nx,
+                              uint64_t ny, int sched, uint64_t chunk, uint32_t teams,
+                              uint32_t threads) {
+  const WindowPlan none = {0, 0, 0u};
+  const bool whole = sched == kStatic, odd = nx % 4 != 0;
+  const uint64_t n = nx * ny;
+  if ((!whole && sched != kChunked && sched != kDynamic && sched != kNonmono) || n == 0 ||
+      nx >= (1ull << 24) || ny >= (1ull << 31) || !aligned)
+    return none;
+  const uint64_t block = (n - 1) / teams + 1, piece = whole ? block / threads : chunk;
+  if (piece < (whole ? 16u : 8u) || block > (1ull << 24) ||
+      (block < 1024 && (!odd || piece < 32)))
+    return none;
+  // block, rounded to sectors on both sides, a row and a sector on each side
+  WindowPlan p;
+  p.lead = (uint32_t)((nx + 7) / 8 * 8 + 8);
+  p.floats = block + 16 + 2 * (uint64_t)p.lead + 8;
+  p.smem = (size_t)(p.floats + 3) / 4 * 16;
+  if ((int64_t)p.smem > budget) return none;
+  return window_gain(c, nx, n, sched, chunk, piece, teams, threads, p.smem) ? p : none;
+}
+
 // schedule(auto) 2-D stencil by strips of 64 columns a warp (k_stencil_cols.cu),
 // for grids the tensor tiles do not take; the others run in the region kernel.
 //   - Strips at least 0.4 full: the lanes beyond a narrow grid's columns idle

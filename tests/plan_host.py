@@ -33,6 +33,11 @@ int tiles(uint64_t stack, uint64_t n, uint64_t nseg, int dot, uint32_t teams, ui
 int uneven(uint64_t n, int sched, uint32_t teams, uint32_t threads) {
   return overlap_uneven(n, sched, teams, threads, 152);
 }
+int window(int64_t budget, uint64_t nx, uint64_t ny, int sched, uint64_t chunk, uint32_t teams,
+           uint32_t threads) {
+  return window_plan({152, 232448, 233472, 32768}, budget, true, nx, ny, sched, chunk, teams,
+                     threads).smem != 0;
+}
 int cols(uint64_t nx, uint64_t ny, uint32_t teams, uint32_t threads) {
   return cols_applies(nx, ny, teams, threads);
 }
@@ -99,3 +104,9 @@ def tiles(n, nseg, teams, threads, single_dot=False, stack=4096):
 def uneven(n, sched, teams, threads):
     """Whether the region kernel's 2-D stencil goes without launch overlap."""
     return bool(_lib().uneven(C.c_uint64(n), sched, C.c_uint32(teams), C.c_uint32(threads)))
+
+
+def window(nx, ny, sched, chunk, teams, threads, budget=232448 - 2048):
+    """Whether a 2-D stencil that none of the forms before takes goes by block windows."""
+    return bool(_lib().window(C.c_int64(budget), C.c_uint64(nx), C.c_uint64(ny), sched,
+                              C.c_uint64(chunk), C.c_uint32(teams), C.c_uint32(threads)))

@@ -143,3 +143,30 @@ def test_generic_tile_rings_fit():
 ])
 def test_stencil2d_launch_overlap(n, sched, G, T, plain):
     assert P.uneven(n, sched, G, T) == plain
+
+
+@pytest.mark.parametrize("nx,ny,sched,chunk,G,T,window", [  # the others and windows in us
+    (4096, 4096, P.CHUNKED, 8, 8192, 32, False),       # 36, 88
+    (4096, 4096, P.CHUNKED, 8, 1024, 32, False),       # 90, 176
+    (2048, 2048, P.STATIC, 0, 4096, 64, False),        # 12, 20
+    (4096, 4096, P.DYNAMIC, 100, 8192, 32, False),     # 45, 74
+    (4096, 4096, P.DYNAMIC, 256, 8192, 32, False),     # 53, 96
+    (4096, 4096, P.DYNAMIC, 256, 16_000, 32, False),   # 105, 158
+    (4096, 4096, P.DYNAMIC, 100, 2048, 32, False),     # 41, 74
+    (4096, 4096, P.NONMONO, 100, 16_000, 32, False),   # 81, 111
+    (16, 306_391, P.DYNAMIC, 1000, 1091, 64, False),   # 52, 99
+    (2048, 39, P.DYNAMIC, 1000, 39, 32, False),        # 14, 27
+    (5, 1737, P.DYNAMIC, 32, 3378, 256, False),        # 13.7, 21.4
+    (3, 444_749, P.CHUNKED, 8, 864, 1024, False),      # 17.0, 24.1
+    (4096, 47, P.CHUNKED, 16, 188, 1024, False),       # 6.5, 9.0
+    (4096, 4096, P.CHUNKED, 64, 608, 256, True),       # 65, 52
+    (4096, 4096, P.STATIC, 0, 608, 256, True),         # 59, 38
+    (4096, 4096, P.DYNAMIC, 256, 608, 256, True),      # 64, 49
+    (3001, 2503, P.CHUNKED, 61, 608, 256, True),       # 37, 24
+    (4096, 4096, P.CHUNKED, 64, 16_000, 32, True),     # 252, 96
+    (7343, 40, P.CHUNKED, 500, 738, 1024, True),       # 382, 67
+    (6054, 913, P.CHUNKED, 16, 565, 1024, True),       # 71, 37
+])
+def test_stencil2d_windows_where_they_gain(nx, ny, sched, chunk, G, T, window):
+    assert P.window(nx, ny, sched, chunk, G, T) == window
+    assert not P.window(nx, ny, sched, chunk, G, T, budget=16)
