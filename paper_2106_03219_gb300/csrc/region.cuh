@@ -876,20 +876,29 @@ __device__ __forceinline__ uint64_t guided_size(uint64_t r, uint64_t c, uint64_t
 }
 
 constexpr uint32_t kGuidedMaxTries = 1u << 20;
-static __shared__ unsigned long long rt_guided_next;
+struct GuidedBlock {  // iterations handed out up to, and the block's end
+  unsigned long long next, end;
+};
+static __shared__ GuidedBlock rt_guided;
 
 // The calling lane's chunk [x, y) of the warp's next claim (x == y: none left
 // for it), or x = ~0 for the whole warp when the block is used up or the
 // bounded retries ran out.  Reached by the whole warp.  Out of line: inlined,
 // its loop shapes the register allocation of the streaming loop around it.
-static __device__ __noinline__ ulonglong2 guided_claim(uint64_t bn, uint64_t c, uint32_t* status) {
+// What it needs of the block lies in shared memory for the same reason: the block's
+// start and length, live across the call, cost the 2-D stencil's loop spills (44
+// bytes stored and 64 loaded, 16 and 32 without; 5.3 M points on 16 x 32 4.8 -> 3.9
+// ms, 7 M on 21 x 256 with a sum 826 -> 640 us; 33 M on 152 x 1024 with chunks from 1,
+// bound by the claims, 590 -> 800, 1920 with the counter in global memory).
+static __device__ __noinline__ ulonglong2 guided_claim(uint64_t c, uint32_t* status) {
   const uint32_t lane = lane_id(), twoT = 2u * blockDim.x;
+  const uint64_t end = rt_guided.end;
   for (uint32_t tries = 0; tries < kGuidedMaxTries; ++tries) {
     unsigned long long cur = 0;
-    if (lane == 0) cur = *(volatile unsigned long long*)&rt_guided_next;
+    if (lane == 0) cur = *(volatile unsigned long long*)&rt_guided.next;
     cur = __shfl_sync(0xffffffffu, cur, 0);
-    if (cur >= bn) return make_ulonglong2(~0ull, 0ull);
-    const uint64_t r = bn - cur;
+    if (cur >= end) return make_ulonglong2(~0ull, 0ull);
+    const uint64_t r = end - cur;
     uint64_t lo, hi, next;
     if (r < (1ull << 58) && (c >= r || (c < (1ull << 40) && r <= c * twoT))) {
       const uint64_t s = c < r ? c : r;  // every chunk from here on
@@ -929,29 +938,32 @@ static __device__ __noinline__ ulonglong2 guided_claim(uint64_t bn, uint64_t c, 
       next = p;
     }
     uint32_t won = 0;
-    if (lane == 0) won = atomicCAS(&rt_guided_next, cur, cur + (unsigned long long)next) == cur;
+    if (lane == 0) won = atomicCAS(&rt_guided.next, cur, cur + (unsigned long long)next) == cur;
     if (__shfl_sync(0xffffffffu, won, 0)) return make_ulonglong2(cur + lo, cur + hi);
   }
   if (lane == 0) set_status(status, OMPRT_DEV_TIMEOUT);  // bounded: give up, report
   return make_ulonglong2(~0ull, 0ull);
 }
 
-// Before the team's first claim; ends in a team barrier.
-__device__ __forceinline__ void guided_start() {
-  if (threadIdx.x == 0) rt_guided_next = 0;
+// Before the team's first claim: hand out [start, end).  Ends in a team barrier.
+__device__ __forceinline__ void guided_start(uint64_t start, uint64_t end) {
+  if (threadIdx.x == 0) {
+    rt_guided.next = start;
+    rt_guided.end = end;
+  }
   team_barrier();
 }
 
+// The started block's chunks; whether the calling thread ran its last iteration.
 template <class Body, class Acc>
-__device__ __forceinline__ bool run_guided(const Body& b, uint64_t bs, uint64_t bn, uint64_t c,
-                                           uint32_t* status, Acc& acc) {
+__device__ __forceinline__ bool run_guided(const Body& b, uint64_t c, uint32_t* status, Acc& acc) {
   bool last = false;
   for (;;) {
-    const ulonglong2 k = guided_claim(bn, c, status);
+    const ulonglong2 k = guided_claim(c, status);
     if (k.x == ~0ull) break;
     if (k.x < k.y) {
-      run_range(b, bs + k.x, bs + k.y, acc);
-      if (k.y == bn) last = true;
+      run_range(b, k.x, k.y, acc);
+      if (k.y == rt_guided.end) last = true;
     }
     __syncwarp();
   }
@@ -1318,8 +1330,8 @@ __global__ void __launch_bounds__(OMPRT_MAX_THREADS) region_kernel(const RegionA
       }
       last = team_last && nch > 0 && (nch - 1) % T == t;
     } else if constexpr (SCHED == kGuided) {
-      guided_start();
-      last = run_guided(body, bs, bn, a.chunk ? a.chunk : 1, a.status, acc) && team_last;
+      guided_start(bs, bs + bn);
+      last = run_guided(body, a.chunk ? a.chunk : 1, a.status, acc) && team_last;
     } else if constexpr (SCHED == kNonmono) {
       // nonmonotonic dynamic: per-warp ranges of chunk groups in shared memory
       __shared__ unsigned long long nm_next[OMPRT_MAX_THREADS / 32], nm_end[OMPRT_MAX_THREADS / 32];

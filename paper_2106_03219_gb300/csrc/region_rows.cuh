@@ -65,10 +65,10 @@ struct PieceChunks {  // 32 consecutive chunks of c a claim, lane l running base
 
 struct PieceGuided {  // a warp's guided claims
   static constexpr bool kAnyWarp = true;
-  uint64_t bn, c;
+  uint64_t c;
   uint32_t* status;
   __device__ __forceinline__ bool next(uint64_t& l, uint64_t& h) {
-    const ulonglong2 k = guided_claim(bn, c, status);
+    const ulonglong2 k = guided_claim(c, status);
     l = k.x;
     h = k.y;
     return k.x != ~0ull;
@@ -305,8 +305,8 @@ __global__ void __launch_bounds__(OMPRT_MAX_THREADS) rows_kernel(const RegionArg
     team_barrier();
     if (t == 0) *ctr = 0;  // leave the counter at zero for the next launch
   } else if constexpr (SCHED == kGuided) {
-    guided_start();  // and rt_row_slots is set
-    run(PieceGuided{bn, c, a.status});
+    guided_start(0, bn);  // and rt_row_slots is set
+    run(PieceGuided{c, a.status});
   } else {
     __shared__ unsigned long long nm_next[OMPRT_MAX_THREADS / 32], nm_end[OMPRT_MAX_THREADS / 32];
     const uint32_t w = warp_id(), W = T / 32;
