@@ -33,12 +33,13 @@ __device__ __forceinline__ float4 shift4(const float4& a, const float4& b, uint3
   return s & 1 ? make_float4(h.y, h.z, h.w, l) : h;
 }
 
-// the first `bytes` of a unit, the rest of it zero; none if bytes is 0
-__device__ __forceinline__ void cp_async_bytes(uint32_t dst, const char* src, uint32_t bytes) {
+// the first `bytes` of a unit, the rest of it zero
+__device__ __forceinline__ void cp_async_if(bool p, uint32_t dst, const char* src,
+                                            uint32_t bytes) {
   asm volatile(
-      "{ .reg .pred q; setp.ne.u32 q, %2, 0; @q cp.async.cg.shared.global [%0], [%1], 16, %2; }" ::
+      "{ .reg .pred q; setp.ne.u32 q, %2, 0; @q cp.async.cg.shared.global [%0], [%1], 16, %3; }" ::
           "r"(dst),
-      "l"(src), "r"(bytes)
+      "l"(src), "r"((uint32_t)p), "r"(bytes)
       : "memory");
 }
 
@@ -94,13 +95,14 @@ __device__ __forceinline__ void run_stencil_pieces(const BodyStencil2D& b,
                              j0 | j1 << 8, sp.ce | sp.ab << 8 | sp.be << 16 | sp.ae << 24);
       if (j0 < j1) {  // the units beyond the row's NU, each fetched by its lane
         const uint32_t mine = smem_addr(st) + lane * kLane;
-        cp_async_bytes(mine, src - 16, j0 == 0 && row > 0 ? 16 : 0);
-        cp_async_bytes(mine + (NU + 1) * 16, src + RE * 4, centre_bytes(RE, j0, j1, sp.ce));
+        cp_async_if(j0 == 0 && row > 0, mine, src - 16, 16);
+        cp_async_if(centre_fetched(RE, j0, j1, sp.ce), mine + (NU + 1) * 16, src + RE * 4,
+                    unit_bytes(RE, sp.ce));
         if (sn | ss) {
-          cp_async_bytes(mine + kN + NU * 16, src + RE * 4 - up * 4,
-                         above_bytes(RE, j0, j1, sn, sp.ab, sp.ae));
-          cp_async_bytes(mine + kSo + NU * 16, src + RE * 4 + down * 4,
-                         below_bytes(RE, j0, j1, ss, sp.be));
+          cp_async_if(above_fetched(RE, j0, j1, sn, sp.ab), mine + kN + NU * 16,
+                      src + RE * 4 - up * 4, above_bytes(RE, nx, sp.ae));
+          cp_async_if(below_fetched(RE, j0, j1, ss, sp.be), mine + kSo + NU * 16,
+                      src + RE * 4 + down * 4, unit_bytes(RE, sp.be));
         }
       }
       __syncwarp();
@@ -110,13 +112,14 @@ __device__ __forceinline__ void run_stencil_pieces(const BodyStencil2D& b,
         const uint4 m = rec[l];
         const char* const p = (const char*)(((uint64_t)m.y << 32) | m.x) + cu * 16;
         const uint32_t dst = smem_addr(st) + l * kLane + cu * 16;
-        const uint32_t i0 = m.z & 255u, i1 = m.z >> 8;
-        if (i0 < i1) {
-          cp_async_bytes(dst + 16, p, centre_bytes(k4, i0, i1, m.w & 255u));
-          cp_async_bytes(dst + kN, p - up * 4,
-                         above_bytes(k4, i0, i1, sn, m.w >> 8 & 255u, m.w >> 24));
-          cp_async_bytes(dst + kSo, p + down * 4, below_bytes(k4, i0, i1, ss, m.w >> 16 & 255u));
-        }
+        const uint32_t i0 = m.z & 255u, i1 = m.z >> 8, ce = m.w & 255u, ab = m.w >> 8 & 255u,
+                       be = m.w >> 16 & 255u;
+        const bool some = i0 < i1;
+        cp_async_if(some && centre_fetched(k4, i0, i1, ce), dst + 16, p, unit_bytes(k4, ce));
+        cp_async_if(some && above_fetched(k4, i0, i1, sn, ab), dst + kN, p - up * 4,
+                    above_bytes(k4, nx, m.w >> 24));
+        cp_async_if(some && below_fetched(k4, i0, i1, ss, be), dst + kSo, p + down * 4,
+                    unit_bytes(k4, be));
       }
       cp_async_commit();
     }
@@ -253,8 +256,9 @@ __device__ __forceinline__ void run_line_pieces(const BodyStencil1D& b, uint64_t
                            j0 | j1 << 8, ce);
     if (j0 < j1) {  // the units beside the row, each fetched by its lane
       const uint32_t mine = smem_addr(st) + lane * kLane;
-      cp_async_bytes(mine, src - 16, j0 == 0 && row > 0 ? 16 : 0);
-      cp_async_bytes(mine + (NU + 1) * 16, src + RE * 4, centre_bytes(RE, j0, j1, ce));
+      cp_async_if(j0 == 0 && row > 0, mine, src - 16, 16);
+      cp_async_if(centre_fetched(RE, j0, j1, ce), mine + (NU + 1) * 16, src + RE * 4,
+                  unit_bytes(RE, ce));
     }
     __syncwarp();
 #pragma unroll
@@ -262,10 +266,8 @@ __device__ __forceinline__ void run_line_pieces(const BodyStencil1D& b, uint64_t
       const uint32_t l = q * (32 / NU) + cr;
       const uint4 m = rec[l];
       const uint32_t i0 = m.z & 255u, i1 = m.z >> 8;
-      if (i0 < i1)
-        cp_async_bytes(smem_addr(st) + l * kLane + cu * 16 + 16,
-                       (const char*)(((uint64_t)m.y << 32) | m.x) + cu * 16,
-                       centre_bytes(k4, i0, i1, m.w));
+      cp_async_if(i0 < i1 && centre_fetched(k4, i0, i1, m.w), smem_addr(st) + l * kLane + cu * 16 + 16,
+                  (const char*)(((uint64_t)m.y << 32) | m.x) + cu * 16, unit_bytes(k4, m.w));
     }
     cp_async_commit();
     cp_async_wait(0);
@@ -322,7 +324,7 @@ __device__ __forceinline__ void run_line_pieces(const BodyStencil1D& b, uint64_t
   }
 }
 
-constexpr unsigned kPieceThreads = 512;  // largest team: 128 registers a thread
+constexpr unsigned kPieceThreads = 512;  // largest team in two dimensions
 template <int SCHED, uint32_t NU>  // NU 0: the 1-D stencil
 __global__ void __launch_bounds__(NU ? kPieceThreads : 1024)
     stencil_pieces_kernel(const StencilPieceArgs P) {

@@ -20,8 +20,7 @@ static std::vector<char> have;  // element of the grid fetched into the span at 
 static int bad = 0;
 static void fetch(int64_t at, uint32_t bytes, const char* what, uint64_t nx, uint64_t row,
                   uint32_t j0, uint32_t j1) {
-  if (!bytes) return;
-  if (at < 0 || at + bytes / 4 > n || bytes % 4) {
+  if (at < 0 || bytes == 0 || bytes > 16 || at + bytes / 4 > n || bytes % 4) {
     if (++bad < 20)
       printf("%s nx=%llu n=%llu row=%llu [%u,%u): %lld + %u bytes\n", what,
              (unsigned long long)nx, (unsigned long long)n, (unsigned long long)row, j0, j1,
@@ -47,13 +46,13 @@ static void grid(uint64_t nx, uint64_t ny) {
           if (k == 1 && j0 == 0 && row > 0) fetch(row - 4, 16, "left", nx, row, j0, j1);
           for (uint32_t u = 0; u <= RE; u += 4) {
             if (u == RE && k != 1 && !(sn | ss)) continue;
-            if (k == 0)
-              fetch((int64_t)row - (int64_t)up + u, above_bytes(u, j0, j1, sn, s.ab, s.ae), "above",
-                    nx, row, j0, j1);
-            if (k == 1)
-              fetch(row + u, centre_bytes(u, j0, j1, s.ce), "centre", nx, row, j0, j1);
-            if (k == 2)
-              fetch(row + down + u, below_bytes(u, j0, j1, ss, s.be), "below", nx, row, j0, j1);
+            if (k == 0 && above_fetched(u, j0, j1, sn, s.ab))
+              fetch((int64_t)row - (int64_t)up + u, above_bytes(u, nx, s.ae), "above", nx, row, j0,
+                    j1);
+            if (k == 1 && centre_fetched(u, j0, j1, s.ce))
+              fetch(row + u, unit_bytes(u, s.ce), "centre", nx, row, j0, j1);
+            if (k == 2 && below_fetched(u, j0, j1, ss, s.be))
+              fetch(row + down + u, unit_bytes(u, s.be), "below", nx, row, j0, j1);
           }
           span[k] = have;
         }
