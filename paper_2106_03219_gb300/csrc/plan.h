@@ -396,8 +396,10 @@ inline bool overlap_uneven(uint64_t n, int sched, uint32_t teams, uint32_t threa
 //     on 864 x 1024 17.0 -> 24.1), and where blocks and rows are whole 32-byte
 //     sectors, so that the plain form reads vectors: others (static(8), 4096^2 on
 //     8192 x 32 36 -> 88, on 1024 x 32 90 -> 176; static, 16 points a thread, 2048^2 on
-//     4096 x 64 12 -> 20); static(c) of such short pieces also on blocks under 1536
-//     points of large grids (static(16), 4096 x 47 on 188 x 1024 6.5 -> 9.0);
+//     4096 x 64 12 -> 20; but with halos below 0.4 of a block windows: static(16), 8 x
+//     1,741,190 on 9519 x 32 148 -> 53); static(c) of such short pieces also on blocks
+//     under 1536 points with four times the halo (static(16), 4096 x 47 on 188 x 1024
+//     6.5 -> 9.0);
 //   - dynamic on grids of whole units, teams of up to 384 threads: the row ring and
 //     the streamed ring with twelve teams an SM on, but for small halos (4096^2,
 //     dynamic(100) on 8192 x 32 45 -> 74, on 2048 x 128 44 -> 45; dynamic(256) on 16,000
@@ -417,12 +419,12 @@ inline bool window_gain(const PlanDevice& c, uint64_t nx, uint64_t n, int sched,
   const uint64_t block = (n - 1) / teams + 1;
   const bool whole = sched == kStatic, few = piece < 24, odd = nx % 4 != 0;
   if (block < 16 || (few && nx <= 3)) return false;
-  if (few && (whole || sched == kChunked) && nx % 8 == 0 && n % (8ull * teams) == 0 &&
-      (!whole || n % (8ull * teams * threads) == 0))
-    return false;
-  if (few && sched == kChunked && block < 1536 && n > 800000) return false;
   // rows of halo a block, resident CTAs an SM, lanes an SM that get a chunk
   const double halo = 2.0 * (double)nx / (double)block;
+  if (few && (whole || sched == kChunked) && halo >= 0.4 && nx % 8 == 0 &&
+      n % (8ull * teams) == 0 && (!whole || n % (8ull * teams * threads) == 0))
+    return false;
+  if (few && sched == kChunked && block < 1536 && halo >= 4) return false;
   const double fit = std::fmin(std::fmin(threads < 1024 ? 1024 / threads : 1, 32),
                                std::fmax(1, std::floor((double)c.smem_per_sm / (smem + 1624.0))));
   const double resident = std::fmin(fit, std::ceil((double)teams / c.sm_count));

@@ -166,6 +166,9 @@ def test_stencil2d_launch_overlap(n, sched, G, T, plain):
     (4096, 4096, P.CHUNKED, 64, 16_000, 32, True),     # 252, 96
     (7343, 40, P.CHUNKED, 500, 738, 1024, True),       # 382, 67
     (6054, 913, P.CHUNKED, 16, 565, 1024, True),       # 71, 37
+    (8, 1_741_190, P.CHUNKED, 16, 9519, 32, True),     # 148, 53
+    (64, 672, P.CHUNKED, 8, 14, 64, True),             # 13.3, 7.6
+    (25, 33_226, P.CHUNKED, 16, 608, 256, True),       # 10.8, 7.6
 ])
 def test_stencil2d_windows_where_they_gain(nx, ny, sched, chunk, G, T, window):
     assert P.window(nx, ny, sched, chunk, G, T) == window
