@@ -336,7 +336,8 @@ inline LinePlan line_plan(const PlanDevice& c, bool aligned16, uint64_t n, int s
 //     one after another where four plain ones share an SM (161 x 256 31 -> 52, 524 x 256
 //     42 -> 133, 2704 x 256 58 -> 184); up to 128 threads it pays from segments of 16
 //     elements a thread on (1765 x 32, segments of 13,000 418 -> 101, 960 x 128 of 3500
-//     47 -> 30, 3005 x 32 of 100 12 -> 30).
+//     47 -> 30, 3005 x 32 of 100 12 -> 30), and up to two waves where half the teams
+//     have none (1020 x 32, 97 segments 6.8 -> 5.3).
 constexpr uint32_t kTilesMax = 8;
 constexpr uint32_t kTiledThreads = 480;  // largest team, 512 threads with the feeder
 struct TilePlan {
@@ -359,7 +360,8 @@ inline TilePlan tile_plan(const PlanDevice& c, uint32_t stack_bytes, uint64_t n,
   p.tiles = tiles < kTilesMax ? (uint32_t)tiles : kTilesMax;
   const double a_thread = (double)n / (double)nseg / threads;  // a segment's elements
   if (want <= fit) return single_dot && nseg <= teams && a_thread < 1 ? none : p;
-  return threads <= 128 && a_thread >= 16 ? p : none;
+  const bool idle = want <= 2 * fit && nseg <= teams / 2 && !(single_dot && a_thread < 1);
+  return threads <= 128 && (a_thread >= 16 || idle) ? p : none;
 }
 
 // Whether a grid of the region kernel's point-by-point 2-D stencil goes without

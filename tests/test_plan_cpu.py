@@ -114,6 +114,9 @@ def test_stencil1d_pieces_where_they_gain(n, sched, chunk, G, T, pieces):
     (568, 13_000, 1765, 32, False, True),       # 418, 101
     (2370, 3505, 960, 128, False, True),        # 47, 30
     (3906, 7800, 7, 128, False, True),          # 4199, 1407
+    (97, 363, 1020, 32, True, True),            # 6.8, 5.3
+    (132, 369, 906, 64, False, True),           # 8.5, 7.0
+    (2001, 31, 1107, 32, True, False),          # 6.7, 10.9
 ])
 def test_generic_tiles_where_they_gain(nseg, avg, G, T, dot, tiled):
     assert (P.tiles(nseg * avg, nseg, G, T, dot) > 0) == tiled
