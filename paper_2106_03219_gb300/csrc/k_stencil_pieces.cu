@@ -19,6 +19,7 @@ namespace rt {
 struct StencilPieceArgs {
   RegionArgs r;       // n, chunk, x, out, c0, c1, nx, ny, dyn_next
   uint32_t sn, ss;    // elements the rows above / below are off: -nx, nx mod 4
+  uint64_t up;        // how far up the span above starts (piece_spans.h)
 };
 
 __host__ __device__ constexpr uint32_t piece_lane_units(uint32_t nu) { return 3 * nu + 5; }
@@ -62,7 +63,7 @@ __device__ __forceinline__ void run_stencil_pieces(const BodyStencil2D& b,
   const RegionArgs& a = P.r;
   const uint32_t lane = lane_id(), sn = P.sn, ss = P.ss;
   const uint32_t nx = (uint32_t)a.nx, ny = (uint32_t)a.ny;
-  const uint64_t n = a.n, up = a.nx + sn, down = a.nx - ss;
+  const uint64_t n = a.n, up = P.up, down = a.nx - ss;
   unsigned char* st = nullptr;  // this warp's rows, from its first claim on
   uint64_t pos = 0, end = 0;
   const uint32_t cu = lane % NU, cr = lane / NU, k4 = 4 * cu;
@@ -92,16 +93,16 @@ __device__ __forceinline__ void run_stencil_pieces(const BodyStencil2D& b,
       }
       const char* const src = (const char*)(b.in + row);
       rec[lane] = make_uint4((uint32_t)(uintptr_t)src, (uint32_t)((uintptr_t)src >> 32),
-                             j0 | j1 << 8, sp.ce | sp.ab << 8 | sp.be << 16 | sp.ae << 24);
+                             j0 | j1 << 8, sp.ce | sp.ab << 8 | sp.be << 16);
       if (j0 < j1) {  // the units beyond the row's NU, each fetched by its lane
         const uint32_t mine = smem_addr(st) + lane * kLane;
         cp_async_if(j0 == 0 && row > 0, mine, src - 16, 16);
-        cp_async_if(centre_fetched(RE, j0, j1, sp.ce), mine + (NU + 1) * 16, src + RE * 4,
+        cp_async_if(centre_edge(RE, j1, sp.ce), mine + (NU + 1) * 16, src + RE * 4,
                     unit_bytes(RE, sp.ce));
         if (sn | ss) {
-          cp_async_if(above_fetched(RE, j0, j1, sn, sp.ab), mine + kN + NU * 16,
-                      src + RE * 4 - up * 4, above_bytes(RE, nx, sp.ae));
-          cp_async_if(below_fetched(RE, j0, j1, ss, sp.be), mine + kSo + NU * 16,
+          cp_async_if(above_edge(RE, j1, sn, sp.ab), mine + kN + NU * 16,
+                      src + RE * 4 - up * 4, 16);
+          cp_async_if(below_edge(RE, j1, ss, sp.be), mine + kSo + NU * 16,
                       src + RE * 4 + down * 4, unit_bytes(RE, sp.be));
         }
       }
@@ -113,12 +114,10 @@ __device__ __forceinline__ void run_stencil_pieces(const BodyStencil2D& b,
         const char* const p = (const char*)(((uint64_t)m.y << 32) | m.x) + cu * 16;
         const uint32_t dst = smem_addr(st) + l * kLane + cu * 16;
         const uint32_t i0 = m.z & 255u, i1 = m.z >> 8, ce = m.w & 255u, ab = m.w >> 8 & 255u,
-                       be = m.w >> 16 & 255u;
-        const bool some = i0 < i1;
-        cp_async_if(some && centre_fetched(k4, i0, i1, ce), dst + 16, p, unit_bytes(k4, ce));
-        cp_async_if(some && above_fetched(k4, i0, i1, sn, ab), dst + kN, p - up * 4,
-                    above_bytes(k4, nx, m.w >> 24));
-        cp_async_if(some && below_fetched(k4, i0, i1, ss, be), dst + kSo, p + down * 4,
+                       be = m.w >> 16;
+        cp_async_if(centre_fetched(k4, i0, i1, ce), dst + 16, p, unit_bytes(k4, ce));
+        cp_async_if(above_fetched(k4, i0, i1, sn, ab), dst + kN, p - up * 4, 16);
+        cp_async_if(below_fetched(k4, i0, i1, ss, be), dst + kSo, p + down * 4,
                     unit_bytes(k4, be));
       }
       cp_async_commit();
@@ -257,7 +256,7 @@ __device__ __forceinline__ void run_line_pieces(const BodyStencil1D& b, uint64_t
     if (j0 < j1) {  // the units beside the row, each fetched by its lane
       const uint32_t mine = smem_addr(st) + lane * kLane;
       cp_async_if(j0 == 0 && row > 0, mine, src - 16, 16);
-      cp_async_if(centre_fetched(RE, j0, j1, ce), mine + (NU + 1) * 16, src + RE * 4,
+      cp_async_if(centre_edge(RE, j1, ce), mine + (NU + 1) * 16, src + RE * 4,
                   unit_bytes(RE, ce));
     }
     __syncwarp();
@@ -266,7 +265,7 @@ __device__ __forceinline__ void run_line_pieces(const BodyStencil1D& b, uint64_t
       const uint32_t l = q * (32 / NU) + cr;
       const uint4 m = rec[l];
       const uint32_t i0 = m.z & 255u, i1 = m.z >> 8;
-      cp_async_if(i0 < i1 && centre_fetched(k4, i0, i1, m.w), smem_addr(st) + l * kLane + cu * 16 + 16,
+      cp_async_if(centre_fetched(k4, i0, i1, m.w), smem_addr(st) + l * kLane + cu * 16 + 16,
                   (const char*)(((uint64_t)m.y << 32) | m.x) + cu * 16, unit_bytes(k4, m.w));
     }
     cp_async_commit();
@@ -431,7 +430,8 @@ cudaError_t launch_stencil2d_pieces(int sched, unsigned teams, unsigned threads,
   if ((uint64_t)warps * piece_stage_bytes(nu) > room) nu = 4;
   const size_t smem = (size_t)warps * piece_stage_bytes(nu);
   if (smem > room) return cudaErrorNotSupported;
-  const StencilPieceArgs P = {a, (uint32_t)(4 - a.nx % 4) % 4, (uint32_t)(a.nx % 4)};
+  const StencilPieceArgs P = {a, (uint32_t)(4 - a.nx % 4) % 4, (uint32_t)(a.nx % 4),
+                              piece_up(a.nx)};
   switch (sched) {
     case kStatic: return launch_pieces_nu<kStatic>(nu, teams, threads, smem, st, P);
     case kChunked: return launch_pieces_nu<kChunked>(nu, teams, threads, smem, st, P);

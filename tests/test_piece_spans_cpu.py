@@ -3,8 +3,8 @@ kernel's own index arithmetic (csrc/piece_spans.h) over small grids, every row
 position and every piece of a row: no fetch leaves the grid, and every neighbour
 of an inner point is fetched.
 
-A grid one column wide moves the span above by up = 4 for nx = 1, so its last
-unit reaches past the array's last element unless it is cut there."""
+A grid one column wide would move the span above by up = 4 for nx = 1, and its last
+unit would reach past the array's last element: no point needs it, and none is fetched."""
 import subprocess
 
 from paper_2106_03219_gb300 import build_lib
@@ -34,10 +34,10 @@ template <uint32_t RE>
 static void grid(uint64_t nx, uint64_t ny) {
   n = nx * ny;
   const uint32_t sn = (4 - nx % 4) % 4, ss = nx % 4;
-  const uint64_t up = nx + sn, down = nx - ss;
+  const uint64_t up = piece_up(nx), down = nx - ss;
   for (uint64_t row = 0; row < n; row += RE) {
     const PieceSpans s = piece_spans<RE>(row, n, up, down);
-    if (s.ce > 255 || s.ab > 255 || s.ae > 255 || s.be > 255) ++bad;
+    if (s.ce > 255 || s.ab > 255 || s.be > 255) ++bad;
     for (uint32_t j0 = 0; j0 < RE && row + j0 < n; ++j0)
       for (uint32_t j1 = j0 + 1; j1 <= RE && row + j1 <= n; ++j1) {
         std::vector<char> span[3];
@@ -46,12 +46,11 @@ static void grid(uint64_t nx, uint64_t ny) {
           if (k == 1 && j0 == 0 && row > 0) fetch(row - 4, 16, "left", nx, row, j0, j1);
           for (uint32_t u = 0; u <= RE; u += 4) {
             if (u == RE && k != 1 && !(sn | ss)) continue;
-            if (k == 0 && above_fetched(u, j0, j1, sn, s.ab))
-              fetch((int64_t)row - (int64_t)up + u, above_bytes(u, nx, s.ae), "above", nx, row, j0,
-                    j1);
-            if (k == 1 && centre_fetched(u, j0, j1, s.ce))
+            if (k == 0 && (u == RE ? above_edge(RE, j1, sn, s.ab) : above_fetched(u, j0, j1, sn, s.ab)))
+              fetch((int64_t)row - (int64_t)up + u, 16, "above", nx, row, j0, j1);
+            if (k == 1 && (u == RE ? centre_edge(RE, j1, s.ce) : centre_fetched(u, j0, j1, s.ce)))
               fetch(row + u, unit_bytes(u, s.ce), "centre", nx, row, j0, j1);
-            if (k == 2 && below_fetched(u, j0, j1, ss, s.be))
+            if (k == 2 && (u == RE ? below_edge(RE, j1, ss, s.be) : below_fetched(u, j0, j1, ss, s.be)))
               fetch(row + down + u, unit_bytes(u, s.be), "below", nx, row, j0, j1);
           }
           span[k] = have;
