@@ -265,23 +265,28 @@ inline StreamPlan stream_plan(const PlanDevice& c, const StageShape& sh, bool st
 }
 
 // 1-D stencil by lanes' pieces (k_stencil_pieces.cu); smem 0: not this form.
-// A warp's slabs follow one another here too, so it takes many warps, or data
-// from DRAM.  Measured plain -> pieces (us, G x T teams x threads), n of 1177
-// random launches:
+// A warp's slabs follow one another, so it takes data from DRAM or many warps, and
+// pieces that fill their rows: whole 32 points, or 80 on (a piece of 40 touches two or
+// three rows).  Measured plain -> pieces (us, G x T teams x threads) on 1627 random
+// launches; the rule is 5 % and more from the better one in 44 of them:
 //   - chunks of 32 points on in blocks of 32 chunks (n = 2^26, 608 x 256: static(64)
 //     210 -> 129, dynamic(256) 151 -> 143; n = 2^22 dynamic(256), 27 chunks a block:
 //     15.6 -> 16.1), and under static pieces of 64 to 256 points and from 1024 on
 //     (608 x 256: 431 points 123 -> 138; 148 x 128, 3542 points 222 -> 181);
-//   - static: teams of 384 threads, or 26 MB of arrays (a fifth of the L2) and a
-//     warp an SM (26 x 32, 2,356,909 points 58 -> 120);
-//   - static(c): three busy warps a team or 0.6 an SM (static(1000) 3 x 32 220 ->
-//     427, 46 -> 89), for chunks that are no multiple of 32 points 80 points and
-//     five warps or 26 MB, or 29 an SM (static(40) 6 x 64 173 -> 440);
-//   - dynamic and nonmonotonic: seven busy warps a team, or four an SM in blocks of
-//     48 chunks (dynamic(500) 18 x 32 81 -> 167, nonmonotonic(256) 164 x 512, 33
-//     chunks a block 12.3 -> 18.8); chunks that are no multiple of 32 points from 26
-//     MB and eight warps an SM on, 16 below 80 points (dynamic(40) 1 x 64 144 -> 315,
-//     nonmonotonic(50) 662 x 256 n = 67 M 258 -> 162).
+//   - static: 26 MB of arrays (a fifth of the L2), teams of 512 threads, or of 256 with
+//     80 to 128 points or 1024 on (79 x 256, 95 points 11.9 -> 8.2; 4 x 256, 70 points 6.4 ->
+//     7.3);
+//   - whole 32 points: 26 MB (under dynamic and nonmonotonic in blocks of 72 chunks or
+//     48 MB: 5,700,616 points, dynamic(256) 608 x 256, 37 chunks 17 -> 20), five busy
+//     warps a team (dynamic(64), 28 x 128, four, 8 M points 197 -> 158, 50 x 64, two
+//     4.9 -> 5.4), or four an SM at once (dynamic(64), 1.2 M points on 595 x 1024, one
+//     14.7 -> 17.5);
+//   - 80 points on, no multiple of 32: as much data, or more warps, nine under static(c)
+//     (static(500) 1 x 256 37 -> 42), twelve else (dynamic(100) 30 x 1024, six, 7.7 -> 9.3;
+//     dynamic(1000) 1 x 512, sixteen 404 -> 292);
+//   - shorter: 26 MB and sixteen warps an SM (dynamic(40), 608 x 256 180 -> 139, but 133
+//     x 32 237 -> 299), from 45 points on also 40 MB or sixteen warps a team (dynamic(50)
+//     5 x 1024 96 -> 78, 426 x 1024, six 16.6 -> 19.3).
 constexpr uint32_t kLineNu = 8;  // 16-byte units a row
 constexpr uint32_t kLineStage = 32 * 16 * (kLineNu + 4);
 struct LinePlan {
@@ -310,13 +315,15 @@ inline LinePlan line_plan(const PlanDevice& c, bool aligned16, uint64_t n, int s
   const bool dram = n * 8 > 26000000, even = chunk % 32 == 0;
   bool gain;
   if (whole)
-    gain = threads >= 384 || (dram && an_sm >= 1);
+    gain = dram || threads >= 512 ||
+           (threads >= 256 && (piece >= 1024 || (piece >= 80 && piece <= 128)));
+  else if (!even && piece < 80)
+    gain = (dram && (an_sm >= 16 || (piece >= 45 && n > 5000000))) || (piece >= 45 && warps >= 16);
   else if (!claims)
-    gain = even ? warps >= 3 || an_sm > 0.6
-                : (piece >= 80 && (dram || warps >= 5)) || an_sm >= 29;
+    gain = (dram && n > 3400000) || warps >= (even ? 5 : 9) || (even && an_sm > 4);
   else
-    gain = even ? warps >= 7 || (an_sm >= 4 && chunks >= 48)
-                : dram && an_sm >= (piece >= 80 ? 8 : 16);
+    gain = (dram && (chunks >= 72 || n > 6000000)) || warps >= (even ? 5 : 12) ||
+           (even && an_sm > 4 && chunks >= 44);
   return gain ? LinePlan{smem} : none;
 }
 

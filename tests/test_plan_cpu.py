@@ -95,6 +95,15 @@ def test_rows_where_they_gain(body, n, sched, chunk, G, T, rows):
     (1 << 24, P.CHUNKED, 32, 608, 256, True),       # 78, 42
     (1 << 24, P.DYNAMIC, 64, 608, 256, True),       # 58, 36
     (66_684_445, P.NONMONO, 50, 662, 256, True),    # 258, 162
+    (16_870_783, P.DYNAMIC, 40, 133, 32, False),    # 237, 299
+    (502_472, P.DYNAMIC, 100, 30, 1024, False),     # 7.7, 9.3
+    (134_259, P.CHUNKED, 500, 1, 256, False),       # 37.4, 42.3
+    (72_320, P.STATIC, 0, 4, 256, False),           # 6.4, 7.3
+    (1_936_512, P.STATIC, 0, 79, 256, True),        # 11.9, 8.2
+    (8_446_615, P.DYNAMIC, 64, 28, 128, True),      # 197, 158
+    (2_005_184, P.DYNAMIC, 1000, 1, 512, True),     # 404, 292
+    (62_584_413, P.DYNAMIC, 40, 608, 256, True),    # 180, 139
+    (1_500_488, P.DYNAMIC, 50, 5, 1024, True),      # 95.8, 78.0
 ])
 def test_stencil1d_pieces_where_they_gain(n, sched, chunk, G, T, pieces):
     assert P.line(n, sched, chunk, G, T) == pieces
