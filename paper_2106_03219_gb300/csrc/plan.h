@@ -124,7 +124,7 @@ inline bool rows_gain(const StageShape& sh, int sched, uint64_t n, uint64_t chun
   if (sh.writes && !comp_sum) {
     if (whole) return piece >= 400;
     if (guided || even) return true;
-    return claims ? share >= 8192 : piece >= 600 || (dram && an_sm <= 3);
+    return claims ? share >= 8192 : piece >= 600 || (dram && an_sm <= 4);
   }
   if (sh.elem == 2) return !whole && !guided && even && warps >= 6;
   if (whole) return dram && piece >= 640;

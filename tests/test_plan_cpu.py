@@ -72,6 +72,7 @@ def test_blocks_aligned_is_exact(body, elem):
     ("axpy", 50_000_001, P.STATIC, 0, 1184, 256, True),         # 124, 102
     ("axpy_i32_sum", 1 << 20, P.STATIC, 0, 4, 128, True),       # 59.8, 53.7
     ("axpy", 1_447_680, P.GUIDED, 64, 39, 256, True),           # 69.3, 14.6
+    ("axpy", 45_266_466, P.CHUNKED, 50, 231, 64, True),         # 356, 222
     ("dot", 30_055_685, P.DYNAMIC, 128, 18, 512, True),         # 491, 232
     ("load_f32_max", 62_239_855, P.DYNAMIC, 128, 3, 1024, True),  # 3044, 1398
     ("load_i32", 18_047_637, P.DYNAMIC, 4096, 26, 512, True),   # 140, 73
