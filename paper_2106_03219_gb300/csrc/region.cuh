@@ -876,8 +876,8 @@ __device__ __forceinline__ uint64_t guided_size(uint64_t r, uint64_t c, uint64_t
 }
 
 constexpr uint32_t kGuidedMaxTries = 1u << 20;
-struct GuidedBlock {  // iterations handed out up to, and the block's end
-  unsigned long long next, end;
+struct GuidedBlock {  // iterations handed out up to, and the least chunk
+  unsigned long long next, c;
 };
 static __shared__ GuidedBlock rt_guided;
 
@@ -885,14 +885,16 @@ static __shared__ GuidedBlock rt_guided;
 // for it), or x = ~0 for the whole warp when the block is used up or the
 // bounded retries ran out.  Reached by the whole warp.  Out of line: inlined,
 // its loop shapes the register allocation of the streaming loop around it.
-// What it needs of the block lies in shared memory for the same reason: the block's
-// start and length, live across the call, cost the 2-D stencil's loop spills (44
-// bytes stored and 64 loaded, 16 and 32 without; 5.3 M points on 16 x 32 4.8 -> 3.9
-// ms, 7 M on 21 x 256 with a sum 826 -> 640 us; 33 M on 152 x 1024 with chunks from 1,
-// bound by the claims, 590 -> 800, 1920 with the counter in global memory).
-static __device__ __noinline__ ulonglong2 guided_claim(uint64_t c, uint32_t* status) {
+// Positions count from the loop's start and the least chunk lies in shared memory for
+// the same reason: the block's start, length and chunk, live across the call, cost the
+// 2-D stencil's loop spills (44 bytes stored and 64 loaded, 20 and 36 without; 5.3 M
+// points on 16 x 32 4.7 -> 3.9 ms, 7 M on 21 x 256 with a sum 826 -> 671 us, 33 M on
+// 152 x 1024 with chunks from 1 586 -> 569).  With the block's end there too, 16 and 32
+// bytes: long chunks 6 % faster still (3.7 ms, 572 us), but its load, first in every
+// claim, holds those of short ones (798 us).
+static __device__ __noinline__ ulonglong2 guided_claim(uint64_t end, uint32_t* status) {
   const uint32_t lane = lane_id(), twoT = 2u * blockDim.x;
-  const uint64_t end = rt_guided.end;
+  const uint64_t c = rt_guided.c;
   for (uint32_t tries = 0; tries < kGuidedMaxTries; ++tries) {
     unsigned long long cur = 0;
     if (lane == 0) cur = *(volatile unsigned long long*)&rt_guided.next;
@@ -946,24 +948,24 @@ static __device__ __noinline__ ulonglong2 guided_claim(uint64_t c, uint32_t* sta
 }
 
 // Before the team's first claim: hand out [start, end).  Ends in a team barrier.
-__device__ __forceinline__ void guided_start(uint64_t start, uint64_t end) {
+__device__ __forceinline__ void guided_start(uint64_t start, uint64_t c) {
   if (threadIdx.x == 0) {
     rt_guided.next = start;
-    rt_guided.end = end;
+    rt_guided.c = c;
   }
   team_barrier();
 }
 
 // The started block's chunks; whether the calling thread ran its last iteration.
 template <class Body, class Acc>
-__device__ __forceinline__ bool run_guided(const Body& b, uint64_t c, uint32_t* status, Acc& acc) {
+__device__ __forceinline__ bool run_guided(const Body& b, uint64_t end, uint32_t* status, Acc& acc) {
   bool last = false;
   for (;;) {
-    const ulonglong2 k = guided_claim(c, status);
+    const ulonglong2 k = guided_claim(end, status);
     if (k.x == ~0ull) break;
     if (k.x < k.y) {
       run_range(b, k.x, k.y, acc);
-      if (k.y == rt_guided.end) last = true;
+      if (k.y == end) last = true;
     }
     __syncwarp();
   }
@@ -1330,8 +1332,8 @@ __global__ void __launch_bounds__(OMPRT_MAX_THREADS) region_kernel(const RegionA
       }
       last = team_last && nch > 0 && (nch - 1) % T == t;
     } else if constexpr (SCHED == kGuided) {
-      guided_start(bs, bs + bn);
-      last = run_guided(body, a.chunk ? a.chunk : 1, a.status, acc) && team_last;
+      guided_start(bs, a.chunk ? a.chunk : 1);
+      last = run_guided(body, bs + bn, a.status, acc) && team_last;
     } else if constexpr (SCHED == kNonmono) {
       // nonmonotonic dynamic: per-warp ranges of chunk groups in shared memory
       __shared__ unsigned long long nm_next[OMPRT_MAX_THREADS / 32], nm_end[OMPRT_MAX_THREADS / 32];

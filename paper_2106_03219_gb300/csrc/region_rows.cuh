@@ -16,9 +16,10 @@
 // Two or more stages a warp: the next slabs load while one is computed (608
 // x 256: 139 us with two stages and 8 warps an SM, 153 with one and 16).
 // Measured, plain -> rows, axpy fp32: dynamic(256) 608 x 256 at n = 2^26 197 ->
-// 135 us (0.89 of the copy rate), static 1184 x 256 at n = 50,000,001 124 ->
-// 102 us (0.87), static(64) 900 x 128 261 -> 142 us, dynamic(256) 608 x 256 at
-// n = 2^22 19.2 -> 12.9 us.  What bounds it now: 128-byte accesses that open a
+// 130-137 us (0.88-0.92 of the copy rate), static 1184 x 256 at n = 50,000,001
+// 124 -> 102-105 us (0.85-0.88), static(64) 900 x 128 261 -> 142 us, dynamic(256) 608 x 256 at
+// n = 2^22 19.2 -> 12.9 us; where it loses, and stays off: rows_gain in plan.h.  What
+// bounds it now: 128-byte accesses that open a
 // DRAM page for each row (whole contiguous windows of a warp's range reached
 // 0.96 under static, but keep only a few lanes busy and lost everywhere
 // else), one-stage teams of 512 and 1024, and the last wave of CTAs.
@@ -65,10 +66,10 @@ struct PieceChunks {  // 32 consecutive chunks of c a claim, lane l running base
 
 struct PieceGuided {  // a warp's guided claims
   static constexpr bool kAnyWarp = true;
-  uint64_t c;
+  uint64_t bn;
   uint32_t* status;
   __device__ __forceinline__ bool next(uint64_t& l, uint64_t& h) {
-    const ulonglong2 k = guided_claim(c, status);
+    const ulonglong2 k = guided_claim(bn, status);
     l = k.x;
     h = k.y;
     return k.x != ~0ull;
@@ -305,8 +306,8 @@ __global__ void __launch_bounds__(OMPRT_MAX_THREADS) rows_kernel(const RegionArg
     team_barrier();
     if (t == 0) *ctr = 0;  // leave the counter at zero for the next launch
   } else if constexpr (SCHED == kGuided) {
-    guided_start(0, bn);  // and rt_row_slots is set
-    run(PieceGuided{c, a.status});
+    guided_start(0, c);  // and rt_row_slots is set
+    run(PieceGuided{bn, a.status});
   } else {
     __shared__ unsigned long long nm_next[OMPRT_MAX_THREADS / 32], nm_end[OMPRT_MAX_THREADS / 32];
     const uint32_t w = warp_id(), W = T / 32;
