@@ -206,17 +206,22 @@ omprt_status omprt_alloc_shared(omprt_ctx *ctx, size_t bytes_per_team);
  * reaches one element / one row beyond the pass, when the chunk is at most
  * 512 bytes and the two halos at most a quarter of the pass.  A claim of 32
  * chunks runs in equal passes.  Streaming bodies whose blocks do not all
- * start on a 16-byte boundary, or whose passes do not fit, take the row form
- * where their pieces are long enough (128 bytes under static(c), dynamic(c) and
- * guided(c), 256 under static): each lane's next 64 or 128 bytes of its piece
+ * start on a 16-byte boundary, or whose passes do not fit, may take the row form
+ * from pieces of 128 bytes on under static(c), dynamic(c), nonmonotonic and
+ * guided(c), of 256 under static: each lane's next 64 or 128 bytes of its piece
  * at a time, in buffers sized from the device's shared memory, whatever
- * `bytes`.  Other launches run the plain form.  The 2-D stencil under
+ * `bytes`.  The 1-D stencil outside the staged form may likewise stage each
+ * lane's next 32 points.  Both run only where they measured faster than the plain
+ * form; the rules, with the figures, are row_plan and line_plan in csrc/plan.h.
+ * Other launches run the plain form.  The 2-D stencil under
  * static(c) with c in [4, 8) or [32, 128] (fp32, no reduction, nx a multiple of
- * 4, n < 2^32, 16-byte-aligned pointers) instead walks each team's block in
+ * 4, n < 2^32, 16-byte-aligned pointers), where the block windows of
+ * omprt_set_stencil_stage_bytes do not take it, walks each team's block in
  * passes of two rows through a six-row ring in shared memory (six rows of nx
  * floats, which must fit the device's per-block shared memory, whatever
  * `bytes`); every thread still runs exactly its own chunks.  bytes is rounded
- * down to 16; 0 turns every staged form, the row ring included, off; more than
+ * down to 16; 0 turns these forms (staged passes, rows, 1-D lane pieces, the
+ * row ring) off; more than
  * the device's per-block shared memory is OMPRT_ERR_INVALID.  Default after
  * init: 32 KiB. */
 omprt_status omprt_set_stage_bytes(omprt_ctx *ctx, int64_t bytes_per_team);
@@ -237,10 +242,12 @@ omprt_status omprt_set_stage_bytes(omprt_ctx *ctx, int64_t bytes_per_team);
  * nx is a multiple of 4, n < 2^32, both pointers are 16-byte aligned,
  * thread_limit <= 512 and the ring holds one team's rows with room to spare.
  * Launches whose blocks or rows line up with nothing (any nx, static, static(c),
- * dynamic(c), nonmonotonic) hold a team's whole block and one row on each side
- * where that fits `bytes`, else stage each thread's next points with the rows
- * above and below; other launches run the forms of omprt_set_stage_bytes.  bytes is rounded
- * down to 16; 0 turns this form off, and with it the slab, band and column-ring
+ * dynamic(c), nonmonotonic) may hold a team's whole block and one row on each
+ * side where that fits `bytes` (window_plan in csrc/plan.h), else stage each
+ * thread's next points with the rows above and below, in buffers sized from the
+ * device's shared memory, however small a non-zero `bytes`; other launches run
+ * the forms of omprt_set_stage_bytes.  bytes is rounded
+ * down to 16; 0 turns all of these off, and with them the slab, band and column-ring
  * forms of omprt_set_stencil_slab_shape and the row ring of
  * dynamic(c) (those size their buffers from the device's shared memory);
  * more than the device's per-block shared memory is OMPRT_ERR_INVALID.
@@ -329,8 +336,9 @@ omprt_status omprt_launch_region_dist(omprt_ctx *ctx, const omprt_loop_desc *des
  * thread dispatches on the id and runs the region's parallel for (the
  * default schedule: static with a chunk of one 32-byte vector, or of one
  * 16-byte unit where the team streams its segments through tiles in the
- * shared memory its stack leaves: teams of up to 480 threads, x and y 16-byte
- * aligned) with a compensated reduction into the variable; a join barrier
+ * shared memory its stack leaves: x and y 16-byte aligned, and all teams resident
+ * at once or small teams with long segments, tile_plan in csrc/plan.h) with a
+ * compensated reduction into the variable; a join barrier
  * returns control to the main thread.  Globalised variables live on the team stack of capacity
  * S (omprt_alloc_shared), overflowing to the team's 4 KiB pool slice (teams
  * below OMPRT_MAX_RED_TEAMS); a request that does not fit sets

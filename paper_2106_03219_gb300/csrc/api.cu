@@ -359,6 +359,7 @@ static omprt_status launch_region_impl(omprt_ctx* c, const omprt_loop_desc* d, i
     const uint64_t cap = 4ull * (uint64_t)c->sm_count;
     teams = (int32_t)(want < 1 ? 1 : (want > cap ? cap : want));
   }
+  // (guided claims in shared memory, but stays limited as when its counters were global)
   const bool counters = ksched == kDynamic || ksched == kGuided;
   if ((acc != kAccNone || counters) && teams > OMPRT_MAX_RED_TEAMS) return OMPRT_ERR_INVALID;
 

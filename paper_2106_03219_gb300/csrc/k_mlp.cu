@@ -9,8 +9,8 @@
 // CTAs' partials in CTA order (deterministic, no atomics).  Both, and the Adam
 // step, overlap the launch before them.
 // Measured, batch 256 (one sample a warp and one thread a parameter walking the
-// batch -> now): under ncu 10.3 + 57.3 -> 7.0 + 3.0 us; a step with Adam through
-// the Python binding 43 -> 19.4 us, what the two host calls take; batch 2048
+// batch -> now): under ncu 10.3 + 57.3 -> 8.6 + 4.4 us; a step with Adam through
+// the Python binding 43 -> 10 us, what the two host calls take; batch 2048
 // 226 -> 19.4, batch 16000 1666 -> 66 us.
 #include <cmath>
 
