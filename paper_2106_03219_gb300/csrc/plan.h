@@ -409,6 +409,14 @@ inline bool overlap_uneven(uint64_t n, int sched, uint32_t teams, uint32_t threa
 //     1,741,190 on 9519 x 32 148 -> 53); static(c) of such short pieces also on blocks
 //     under 1536 points with four times the halo (static(16), 4096 x 47 on 188 x 1024
 //     6.5 -> 9.0);
+//   - static(c), c from 32 to 63, where the windows an SM holds at once have at most two
+//     warps, in more than one wave: lane pieces on odd grids but for the chunks of whole
+//     sectors beyond 32, whose lanes spread over the banks (static(32), 289 x 16,457 on
+//     163 x 32 127 -> 180, static(61), 5369 x 3082 on 700 x 32 106 -> 229; static(40), 847 x
+//     6781 on 181 x 32 148 -> 102); the row ring up to c = 39 on rows of 2048 to 4999 points
+//     (static(32), 2548 x 5652 on 276 x 32 147 -> 250; 192 x 61,956 on 265 x 64 327 -> 127,
+//     5536 x 2774 on 897 x 32 193 -> 119, static(44), 5236 x 1843 on 554 x 32 146 -> 77).
+//     Of 128 random launches of this kind it is the slower choice in 3;
 //   - dynamic on grids of whole units, teams of up to 384 threads: the row ring and
 //     the streamed ring with twelve teams an SM on, but for small halos (4096^2,
 //     dynamic(100) on 8192 x 32 45 -> 74, on 2048 x 128 44 -> 45; dynamic(256) on 16,000
@@ -438,6 +446,10 @@ inline bool window_gain(const PlanDevice& c, uint64_t nx, uint64_t n, int sched,
                                std::fmax(1, std::floor((double)c.smem_per_sm / (smem + 1624.0))));
   const double resident = std::fmin(fit, std::ceil((double)teams / c.sm_count));
   if (sched == kNonmono) return halo <= 6 || teams <= 5 * c.sm_count * fit;
+  if (sched == kChunked && chunk >= 32 && chunk < 64 && fit * threads <= 64 &&
+      teams > c.sm_count * fit &&
+      (odd ? chunk % 8 || chunk == 32 : chunk < 40 && nx >= 2048 && nx < 5000))
+    return false;
   if (sched != kDynamic || odd || threads > 384) return true;
   if (teams > 12u * (uint32_t)c.sm_count) return threads >= 64 && halo <= 1.5;
   const uint64_t chunks = (block - 1) / chunk + 1;

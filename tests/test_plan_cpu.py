@@ -180,6 +180,15 @@ def test_stencil2d_launch_overlap(n, sched, G, T, plain):
     (7343, 40, P.CHUNKED, 500, 738, 1024, True),       # 382, 67
     (6054, 913, P.CHUNKED, 16, 565, 1024, True),       # 71, 37
     (8, 1_741_190, P.CHUNKED, 16, 9519, 32, True),     # 148, 53
+    (2548, 5652, P.CHUNKED, 32, 276, 32, False),       # 147, 250
+    (2393, 6233, P.CHUNKED, 32, 297, 64, False),       # 109, 146
+    (5798, 2480, P.CHUNKED, 32, 596, 32, False),       # 102, 269
+    (847, 6781, P.CHUNKED, 40, 181, 32, True),         # 149, 102
+    (5536, 2774, P.CHUNKED, 32, 897, 32, True),        # 193, 119
+    (192, 61_956, P.CHUNKED, 32, 265, 64, True),       # 327, 127
+    (5088, 1655, P.CHUNKED, 61, 628, 32, True),        # 141, 71
+    (4, 2_597_540, P.CHUNKED, 50, 220, 32, True),      # 7989, 205
+    (174, 68_534, P.CHUNKED, 256, 219, 128, True),     # 69, 52
     (64, 672, P.CHUNKED, 8, 14, 64, True),             # 13.3, 7.6
     (25, 33_226, P.CHUNKED, 16, 608, 256, True),       # 10.8, 7.6
 ])
